@@ -198,6 +198,7 @@ struct TreeIO {
   float* s_cent;    // smem [n_nodes][d]
   int* s_mask;      // smem [n_nodes]
   int bracket;      // 1: the FP32 factors (the directions') scaled by each node's bounding radius
+  int vb;           // threads whose points and order the FP32 sums follow (<= blockDim.x)
 };
 
 // This thread's largest squared Mahalanobis distance, over the live points
@@ -222,6 +223,8 @@ static __device__ __noinline__ unsigned max_mahalanobis2(const float* __restrict
 }
 
 inline __device__ __noinline__ void cluster_tree(const TreeIO& io, const TreeScratch& T, BlockScratch& S, int nw_chol) {
+  // threads that add points (io.vb of them: blocks of any size add them in the same order)
+  const int VB = io.vb, vt = (int)threadIdx.x < VB ? (int)threadIdx.x : io.N;
   const int tid = threadIdx.x, B = blockDim.x, lane = tid & 31, wid = tid >> 5;
   const int d = io.d, N = io.N, D = io.depth, n_nodes = (1 << (D + 1)) - 1;
   const int n_leaves = 1 << D;
@@ -342,7 +345,7 @@ inline __device__ __noinline__ void cluster_tree(const TreeIO& io, const TreeScr
           float acc[kRedW];
 #pragma unroll
           for (int k = 0; k < kRedW; ++k) acc[k] = 0.f;
-          for (int j = tid; j < N; j += B) {
+          for (int j = vt; j < N; j += VB) {
             const int bits = io.side[j];
             const int slot = 2 * (node_at(bits, lev) - first) + ((bits >> lev) & 1) - s0;
             float v4[4];
@@ -384,7 +387,7 @@ inline __device__ __noinline__ void cluster_tree(const TreeIO& io, const TreeScr
       float acc[kRedW];
 #pragma unroll
       for (int k = 0; k < kRedW; ++k) acc[k] = 0.f;
-      for (int j = tid; j < N; j += B) {
+      for (int j = vt; j < N; j += VB) {
         const int lf = node_at(io.side[j], D) - last_first - l0;
         float v8[8];
 #pragma unroll
@@ -424,7 +427,7 @@ inline __device__ __noinline__ void cluster_tree(const TreeIO& io, const TreeScr
         ea[k] = a;
         eb[k] = e - a * (a + 1) / 2;
       }
-      for (int j = tid; j < N; j += B) {
+      for (int j = vt; j < N; j += VB) {
         const int lf = node_at(io.side[j], D) - last_first - l0;
         if (lf < 0 || lf >= kLf) continue;
         float p8[8];

@@ -145,123 +145,123 @@ __device__ __forceinline__ bool candidate(const float (&x)[DMAX], const float (&
   return (mn >= 0.f) && (mx <= 1.f);
 }
 
-// logL at the unit-cube point u (zero beyond d).  Pairs of coordinates (and
-// pairs of rows of L^T) go through one packed FMA each.
-template <int DMAX>
-__device__ __forceinline__ float loglike_u(const LikParams& P, const float (&u)[DMAX]) {
-  float ll;
-  switch (P.kind) {
-    case kIso: {
-      float2 acc = f2(0.f, 0.f);
+// logL at the unit-cube point u (zero beyond d) for one likelihood family.
+// Pairs of coordinates (and pairs of rows of L^T) go through one packed FMA
+// each.
+template <int DMAX, int KIND>
+__device__ __forceinline__ float loglike_k(const LikParams& P, const float (&u)[DMAX]) {
+  float ll = -CUDART_INF_F;
+  if constexpr (KIND == kIso) {
+    float2 acc = f2(0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < DMAX; i += 2) {
-        const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.c + i));
-        acc = __ffma2_rn(y, y, acc);
-      }
-      ll = -(acc.x + acc.y) * P.inv2s2;
-      break;
+    for (int i = 0; i < DMAX; i += 2) {
+      const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.c + i));
+      acc = __ffma2_rn(y, y, acc);
     }
-    case kCorr: {
-      float y[DMAX];
+    ll = -(acc.x + acc.y) * P.inv2s2;
+  } else if constexpr (KIND == kCorr) {
+    float y[DMAX];
 #pragma unroll
-      for (int i = 0; i < DMAX; i += 2) {
-        const float2 q = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.c + i));
-        y[i] = q.x;
-        y[i + 1] = q.y;
-      }
-      float2 acc = f2(0.f, 0.f);
-#pragma unroll
-      for (int jp = 0; jp < DMAX / 2; ++jp) {
-        // (z_{2jp}, z_{2jp+1}) = sum_{i >= 2jp} (L[i][2jp], L[i][2jp+1]) y_i
-        float2 z = f2(0.f, 0.f);
-#pragma unroll
-        for (int i = 2 * jp; i < DMAX; ++i) z = __ffma2_rn(P.LpP[jp * kMaxDim + i], f2(y[i], y[i]), z);
-        acc = __ffma2_rn(z, z, acc);
-      }
-      ll = -0.5f * (acc.x + acc.y);
-      break;
+    for (int i = 0; i < DMAX; i += 2) {
+      const float2 q = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.c + i));
+      y[i] = q.x;
+      y[i + 1] = q.y;
     }
-    case kRosen: {
-      float th[DMAX];
+    float2 acc = f2(0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < DMAX; i += 2) {
-        const float2 q = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.lo + i));
-        th[i] = q.x;
-        th[i + 1] = q.y;
-      }
-      float s = 0.f;
+    for (int jp = 0; jp < DMAX / 2; ++jp) {
+      // (z_{2jp}, z_{2jp+1}) = sum_{i >= 2jp} (L[i][2jp], L[i][2jp+1]) y_i
+      float2 z = f2(0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i + 1 < DMAX; ++i) {
-        const float p = P.a - th[i];
-        const float q = fmaf(-th[i], th[i], th[i + 1]);
-        s = fmaf(P.rw[i], fmaf(p, p, P.b * q * q), s);
-      }
-      ll = -s;
-      break;
+      for (int i = 2 * jp; i < DMAX; ++i) z = __ffma2_rn(P.LpP[jp * kMaxDim + i], f2(y[i], y[i]), z);
+      acc = __ffma2_rn(z, z, acc);
     }
-    case kMix: {
-      float e[kMaxModes];
-      float emax = -CUDART_INF_F;
+    ll = -0.5f * (acc.x + acc.y);
+  } else if constexpr (KIND == kRosen) {
+    float th[DMAX];
 #pragma unroll
-      for (int k = 0; k < kMaxModes; ++k) {
-        e[k] = -CUDART_INF_F;
-        if (k < P.n_modes) {
-          float2 acc = f2(0.f, 0.f);
-#pragma unroll
-          for (int i = 0; i < DMAX; i += 2) {
-            const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.cm + k * kMaxDim + i));
-            acc = __ffma2_rn(y, y, acc);
-          }
-          e[k] = -(acc.x + acc.y) * P.inv2s2;
-          emax = fmaxf(emax, e[k]);
-        }
-      }
-      float acc = 0.f;
-#pragma unroll
-      for (int k = 0; k < kMaxModes; ++k)
-        if (k < P.n_modes) acc += expf(e[k] - emax);
-      ll = emax + logf(acc) - P.log_k;
-      break;
+    for (int i = 0; i < DMAX; i += 2) {
+      const float2 q = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.lo + i));
+      th[i] = q.x;
+      th[i + 1] = q.y;
     }
-    case kGmm: {
-      // log sum_k w_k exp(-sum_i (theta_i - mu_ki)^2 / (2 s_ki^2)), online
-      // max-shifted sum over the modes
-      float mx = -CUDART_INF_F, acc = 0.f;
-      for (int k = 0; k < P.n_modes; ++k) {
-        const float* g = P.gm + k * DMAX;
-        const float* w = P.giv + k * DMAX;
-        float2 s = f2(0.f, 0.f);
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i + 1 < DMAX; ++i) {
+      const float p = P.a - th[i];
+      const float q = fmaf(-th[i], th[i], th[i + 1]);
+      s = fmaf(P.rw[i], fmaf(p, p, P.b * q * q), s);
+    }
+    ll = -s;
+  } else if constexpr (KIND == kMix) {
+    float e[kMaxModes];
+    float emax = -CUDART_INF_F;
+#pragma unroll
+    for (int k = 0; k < kMaxModes; ++k) {
+      e[k] = -CUDART_INF_F;
+      if (k < P.n_modes) {
+        float2 acc = f2(0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < DMAX; i += 2) {
-          const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(g + i));
-          s = __ffma2_rn(__fmul2_rn(y, ld2(w + i)), y, s);
+          const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.cm + k * kMaxDim + i));
+          acc = __ffma2_rn(y, y, acc);
         }
-        const float e = P.glw[k] - (s.x + s.y);
-        if (e > mx) {
-          acc = fmaf(acc, expf(mx - e), 1.f);
-          mx = e;
-        } else {
-          acc += expf(e - mx);
-        }
+        e[k] = -(acc.x + acc.y) * P.inv2s2;
+        emax = fmaxf(emax, e[k]);
       }
-      ll = mx + logf(acc);
-      break;
     }
-    case kShell: {
-      float2 acc = f2(0.f, 0.f);
+    float acc = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMaxModes; ++k)
+      if (k < P.n_modes) acc += expf(e[k] - emax);
+    ll = emax + logf(acc) - P.log_k;
+  } else if constexpr (KIND == kGmm) {
+    // log sum_k w_k exp(-sum_i (theta_i - mu_ki)^2 / (2 s_ki^2)), online
+    // max-shifted sum over the modes
+    float mx = -CUDART_INF_F, acc = 0.f;
+    for (int k = 0; k < P.n_modes; ++k) {
+      const float* g = P.gm + k * DMAX;
+      const float* w = P.giv + k * DMAX;
+      float2 s = f2(0.f, 0.f);
 #pragma unroll
       for (int i = 0; i < DMAX; i += 2) {
-        const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.c + i));
-        acc = __ffma2_rn(y, y, acc);
+        const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(g + i));
+        s = __ffma2_rn(__fmul2_rn(y, ld2(w + i)), y, s);
       }
-      const float z = sqrtf(acc.x + acc.y) - P.a;
-      ll = -z * z * P.inv2s2;
-      break;
+      const float e = P.glw[k] - (s.x + s.y);
+      if (e > mx) {
+        acc = fmaf(acc, expf(mx - e), 1.f);
+        mx = e;
+      } else {
+        acc += expf(e - mx);
+      }
     }
-    default:
-      ll = -CUDART_INF_F;
+    ll = mx + logf(acc);
+  } else if constexpr (KIND == kShell) {
+    float2 acc = f2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < DMAX; i += 2) {
+      const float2 y = __ffma2_rn(ld2(P.span + i), f2(u[i], u[i + 1]), ld2(P.c + i));
+      acc = __ffma2_rn(y, y, acc);
+    }
+    const float z = sqrtf(acc.x + acc.y) - P.a;
+    ll = -z * z * P.inv2s2;
   }
   return (ll != ll) ? -CUDART_INF_F : ll;
+}
+
+// The same for a family known at run time.
+template <int DMAX>
+__device__ __forceinline__ float loglike_u(const LikParams& P, const float (&u)[DMAX]) {
+  switch (P.kind) {
+    case kIso: return loglike_k<DMAX, kIso>(P, u);
+    case kCorr: return loglike_k<DMAX, kCorr>(P, u);
+    case kRosen: return loglike_k<DMAX, kRosen>(P, u);
+    case kMix: return loglike_k<DMAX, kMix>(P, u);
+    case kGmm: return loglike_k<DMAX, kGmm>(P, u);
+    case kShell: return loglike_k<DMAX, kShell>(P, u);
+    default: return -CUDART_INF_F;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -798,6 +798,300 @@ inline __device__ void slice_walker(const LikParams& P, const SliceCfg& S, int w
 }
 
 // ---------------------------------------------------------------------------
+// a5-a7 with one walker per group of G = 2, 4 or 8 lanes (aligned in the
+// warp).  The points a slice step may evaluate are known before any of them
+// is: the stepping-out ends are a, a - w, a - 2 w, .. and b, b + w, .., and a
+// rejected shrink candidate moves the bracket to itself whatever its log L,
+// so candidate k + 1 follows from candidate k alone.  The group's lanes
+// therefore evaluate the next ones at once -- half the lanes on each end
+// while stepping out, then the first shrink candidates -- and the walker
+// takes the outcomes in its own order: it stops an end at the first point
+// outside the slice and takes the first accepted candidate; what lies past
+// that point is dropped, neither counted nor stored.  Each point goes
+// through the same FP32 operations as in slice_walker, so the walk is the
+// same bit for bit; a step takes two to three rounds of likelihoods instead
+// of six or seven.  What that buys depends on idle lanes: a chain of
+// dependent likelihoods is bound by latency, not by lanes, wherever the
+// walkers do not fill the SM.
+//
+// The groups of a warp go in lock step: every group takes its step's ends in
+// one batch, then its first shrink candidates in another, and a further
+// batch follows only while a group of the warp needs one.  A step is then
+// straight code, for one likelihood family at a time: a warp alone on its
+// scheduler pays about five cycles for every instruction, so the instruction
+// count is the time (the same walk as a state machine per group with the
+// family chosen inside it took 5.6 k cycles per step against 2.9 k, 10-D
+// correlated Gaussian, and 3.3 k against 1.4 k at 2 dimensions).
+//
+// Up to 12 dimensions the point, the direction and the next step's row are
+// registers of each lane (mem unused); wider ones keep one copy per group in
+// shared memory, which holds every register class within 128 registers.
+// mem: group_floats(DMAX) floats private to the group, 16-byte aligned: two
+// rows (the step's and the next, copied ahead with cp.async) and x.  All
+// lanes of the warp call it.
+// ---------------------------------------------------------------------------
+__host__ __device__ constexpr int group_xs(int dmax) { return (dmax + 3) & ~3; }
+__host__ __device__ constexpr bool group_in_regs(int dmax) { return dmax <= 12; }
+__host__ __device__ constexpr int group_floats(int dmax) {
+  return group_in_regs(dmax) ? 0 : 2 * dir_row(dmax) + group_xs(dmax);
+}
+
+template <int DMAX, int KIND>
+inline __device__ void slice_walker_lanes(const LikParams& P, const SliceCfg& S, int G, int walker, bool active,
+                                          const float* x0, int x0_stride, float l0, const float* dirs, float* mem,
+                                          float thr_out, float thr_in, const WalkerOut& O, long long& evals_out,
+                                          int& flags_out) {
+  constexpr int RW = dir_row(DMAX), XS = group_xs(DMAX);
+  constexpr bool REG = group_in_regs(DMAX);
+  const int d = S.d, n_steps = S.n_steps, e_max = S.e_max, s_max = S.s_max, t_max = S.t_max;
+  const float width = S.width;
+  const int lane = threadIdx.x & 31, g = lane & (G - 1), base = lane - g, H = G >> 1;
+  const bool right = g >= H;
+  const int je = right ? g - H : g, own0 = right ? base + H : base;  // this lane's side: its place there, first lane
+  const unsigned hones = (1u << H) - 1u, ones = (1u << G) - 1u, gmask = ones << base;
+  const float w = right ? width : -width;
+  float xr[REG ? DMAX : 2], vr[REG ? DMAX : 2];
+  float4 nx[REG ? RW / 4 : 1];
+  float* x = mem + 2 * RW;
+  float* row = mem;
+  float l = l0;
+  int hlen = 0, flags = 0, evals = 0;
+  float r = 0.f, pre[kPreShrink] = {};
+  auto fetch = [&](int s) {  // the row of step s, ahead of its use
+    const float* src = dirs + (size_t)s * RW;
+    if constexpr (REG) {
+#pragma unroll
+      for (int q = 0; q < RW / 4; ++q) nx[q] = *reinterpret_cast<const float4*>(src + 4 * q);
+    } else {
+      for (int q = 4 * g; q < RW; q += 4 * G) cp_async16(mem + (s & 1) * RW + q, src + q);
+      cp_async_commit();
+    }
+  };
+  auto take = [&](int s) {
+    if constexpr (REG) {
+      float f[RW];
+#pragma unroll
+      for (int q = 0; q < RW / 4; ++q) {
+        f[4 * q] = nx[q].x;
+        f[4 * q + 1] = nx[q].y;
+        f[4 * q + 2] = nx[q].z;
+        f[4 * q + 3] = nx[q].w;
+      }
+#pragma unroll
+      for (int i = 0; i < DMAX; ++i) vr[i] = f[i];
+      r = f[DMAX];
+#pragma unroll
+      for (int k = 0; k < kPreShrink; ++k) pre[k] = f[DMAX + 1 + k];
+    } else {
+      row = mem + (s & 1) * RW;
+      cp_async_wait_all();
+      __syncwarp();
+      r = row[DMAX];
+#pragma unroll
+      for (int k = 0; k < kPreShrink; ++k) pre[k] = row[DMAX + 1 + k];
+    }
+  };
+  // the candidate at tp: whether it lies in the cube, its log L
+  auto eval = [&](float tp, float& lp) {
+    float u[DMAX];
+    const float2 t2 = f2(tp, tp);
+#pragma unroll
+    for (int i = 0; i < DMAX; i += 2) {
+      float2 q;
+      if constexpr (REG) q = __ffma2_rn(t2, f2(vr[i], vr[i + 1]), f2(xr[i], xr[i + 1]));
+      else q = __ffma2_rn(t2, ld2(row + i), ld2(x + i));
+      u[i] = q.x;
+      u[i + 1] = q.y;
+    }
+    float mn = u[0], mx = u[0];
+#pragma unroll
+    for (int i = 1; i < DMAX; ++i) {
+      mn = fminf(mn, u[i]);
+      mx = fmaxf(mx, u[i]);
+    }
+    const bool in = (mn >= 0.f) && (mx <= 1.f);
+    if (in) lp = loglike_k<DMAX, KIND>(P, u);
+    return in;
+  };
+  if (active) {
+    if constexpr (REG) {
+#pragma unroll
+      for (int i = 0; i < DMAX; ++i) xr[i] = i < d ? x0[(size_t)i * x0_stride] : 0.f;
+    } else {
+      for (int i = g; i < XS; i += G) x[i] = i < d ? x0[(size_t)i * x0_stride] : 0.f;
+    }
+    if (n_steps > 0) fetch(0);
+  } else if constexpr (REG) {
+#pragma unroll
+    for (int i = 0; i < DMAX; ++i) xr[i] = 0.f;
+#pragma unroll
+    for (int q = 0; q < RW / 4; ++q) nx[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  for (int step = 0; step < n_steps; ++step) {
+    if constexpr (!REG) __syncwarp();
+    take(step);
+    if (active && step + 1 < n_steps) fetch(step + 1);
+    // stepping out: e is this lane's side's end
+    float e = right ? (1.f - r) * width : -r * width;
+    {
+      bool open = active;  // this lane's side is not settled
+      int nexp = 0;
+      do {
+        float tp = e;
+        if (je > 0) tp += w;
+        if (je > 1) tp += w;
+        if (je > 2) tp += w;
+        const bool on = open && nexp + je <= e_max;
+        float lp = -CUDART_INF_F;
+        const bool in = on && eval(tp, lp);
+        const bool ok = in && lp > thr_out;
+        const bool cap = nexp + je >= e_max;
+        const unsigned hb = (__ballot_sync(kFull, on && (!ok || cap)) >> own0) & hones;
+        const unsigned inb = __ballot_sync(kFull, in) >> own0;
+        const int f = hb ? __ffs(hb) - 1 : H - 1;
+        const float te = __shfl_sync(kFull, tp, own0 + f);
+        const bool okf = __shfl_sync(kFull, (int)ok, own0 + f) != 0;
+        if (open) {
+          evals += __popc(inb & ((2u << f) - 1u));  // own side's; added up at the end
+          e = hb ? te : te + w;
+          if (hb && okf) flags |= 1;
+          nexp += H;
+          open = hb == 0;
+        }
+      } while (__any_sync(kFull, open));
+    }
+    float a = __shfl_sync(kFull, e, base), b = __shfl_sync(kFull, e, base + H);
+    // shrinkage: the candidates of a bracket that keeps being rejected
+    bool open = active;
+    int nsh = 0;
+    do {
+      const int K = nsh == 0 ? min(kPreShrink, min(G, s_max)) : min(G, s_max - nsh);
+      float tp = 0.f;
+      float ae = a, be = b;
+      if (nsh == 0) {
+#pragma unroll
+        for (int q = 0; q < kPreShrink; ++q)
+          if (q < K) {
+            const float tq = fmaf(pre[q], be - ae, ae);
+            if (q == g) tp = tq;
+            if (tq < 0.f) ae = tq;
+            else be = tq;
+          }
+      } else {
+        const int k = nsh + g;
+        float uu = 0.f;
+        if (open && g < K)
+          uu = k < kPreShrink
+                   ? (k == 1 ? pre[1] : pre[2])  // (s_max or G may end the first batch early)
+                   : u24(draw_at(S.k0, S.k1, S.t, (uint32_t)walker, (uint32_t)step, shrink_draw0(d) + (uint32_t)k));
+        for (int q = 0; q < G; ++q) {
+          const float tq = fmaf(__shfl_sync(kFull, uu, base + q), be - ae, ae);
+          if (q < K) {
+            if (q == g) tp = tq;
+            if (tq < 0.f) ae = tq;
+            else be = tq;
+          }
+        }
+      }
+      const bool on = open && g < K;
+      float lp = -CUDART_INF_F;
+      const bool in = on && eval(tp, lp);
+      const bool ok = in && lp > thr_in;
+      const unsigned okb = (__ballot_sync(kFull, ok) >> base) & ones;
+      const unsigned inb = __ballot_sync(kFull, in) >> base;
+      const int f = okb ? __ffs(okb) - 1 : K - 1;
+      const float tf = __shfl_sync(kFull, tp, base + f);
+      const float lf = __shfl_sync(kFull, lp, base + f);
+      if (open) {
+        if (g == 0) evals += __popc(inb & ((2u << f) - 1u));
+        if (step == n_steps - 1) {
+          const int k = nsh + g;
+          int hs = -1;
+          if (on && g <= f) hs = k < t_max - 1 ? k : (okb && g == f ? t_max - 1 : -1);
+          if (hs >= 0) {
+            O.hist_l[hs] = lp;
+            float* h = O.hist_x + (size_t)hs * d;
+            if constexpr (REG) {
+#pragma unroll
+              for (int i = 0; i < DMAX; ++i)
+                if (i < d) h[i] = fmaf(tp, vr[i], xr[i]);
+            } else {
+              for (int i = 0; i < d; ++i) h[i] = fmaf(tp, row[i], x[i]);
+            }
+          }
+          const int kl = nsh + f;
+          hlen = kl < t_max - 1 ? kl + 1 : (okb ? t_max : max(hlen, t_max - 1));
+        }
+        if (okb) {  // the accepted point, bit for bit
+          if constexpr (REG) {
+#pragma unroll
+            for (int i = 0; i < DMAX; i += 2) {
+              const float2 q = __ffma2_rn(f2(tf, tf), f2(vr[i], vr[i + 1]), f2(xr[i], xr[i + 1]));
+              xr[i] = q.x;
+              xr[i + 1] = q.y;
+            }
+          } else {
+            __syncwarp(gmask);  // every lane of the group has read x
+            for (int i = g; i < DMAX; i += G) x[i] = fmaf(tf, row[i], x[i]);
+          }
+          l = lf;
+          open = false;
+        } else {
+          a = ae;
+          b = be;
+          if (nsh + K >= s_max) {
+            flags |= 2;
+            open = false;
+          }
+        }
+      }
+      nsh += K;  // the same in every lane of the warp (K is)
+    } while (__any_sync(kFull, open));
+  }
+  if constexpr (!REG) __syncwarp();
+  // the two sides' counts and flags
+  const int ev_r = __shfl_sync(kFull, evals, base + H), fl_r = __shfl_sync(kFull, flags, base + H);
+  evals_out = g == 0 ? evals + ev_r : 0;
+  flags_out = g == 0 ? flags | fl_r : 0;
+  if (active) {
+    if constexpr (REG) {
+      if (g == 0) {
+#pragma unroll
+        for (int i = 0; i < DMAX; ++i)
+          if (i < d) O.new_x[i] = xr[i];
+      }
+    } else {
+      for (int i = g; i < d; i += G) O.new_x[i] = x[i];
+    }
+    if (g == 0) {
+      O.new_l[0] = l;
+      O.hist_len[0] = hlen;
+    }
+  }
+}
+
+// slice_walker_lanes for the run's family.
+template <int DMAX>
+inline __device__ void slice_walker_any(const LikParams& P, const SliceCfg& S, int G, int walker, bool active,
+                                        const float* x0, int x0_stride, float l0, const float* dirs, float* mem,
+                                        float thr_out, float thr_in, const WalkerOut& O, long long& ev, int& fl) {
+#define NS_WALK(KIND)                                                                                             \
+  case KIND:                                                                                                      \
+    slice_walker_lanes<DMAX, KIND>(P, S, G, walker, active, x0, x0_stride, l0, dirs, mem, thr_out, thr_in, O, ev, fl); \
+    return;
+  switch (P.kind) {
+    NS_WALK(kIso)
+    NS_WALK(kCorr)
+    NS_WALK(kRosen)
+    NS_WALK(kMix)
+    NS_WALK(kGmm)
+    NS_WALK(kShell)
+    default: break;
+  }
+#undef NS_WALK
+}
+
+// ---------------------------------------------------------------------------
 // a5-a7 with one walker per warp: the 32 lanes of a warp carry one walker,
 // lane i its coordinate i (d <= 32).  The decisions, draws and history are
 // those of slice_walker; only the order of the FP32 sums inside the
@@ -1180,15 +1474,17 @@ struct EvidState {
 };
 
 inline __device__ void evidence_add(EvidState& E, int N, int n, const float* __restrict__ l_in,
-                             double* logw_out, bool live, BlockScratch& S) {
+                             double* logw_out, bool live, BlockScratch& S, int vb) {
   const double Nd = (double)N;
   const double invN = 1.0 / Nd;
   const double cN = log(-expm1(-invN));
   const double live_off = -(double)E.k * invN - log(Nd);
-  const int tid = threadIdx.x, B = blockDim.x;
+  // the first vb threads take the points (blocks of any size then add them in
+  // the same order)
+  const int tid = threadIdx.x, B = vb, first = tid < vb ? tid : n;
   const long long k0 = E.k;
   double mx = E.logz;
-  for (int j = tid; j < n; j += B) {
+  for (int j = first; j < n; j += B) {
     const double l = (double)l_in[j];
     const double lw = live ? l + live_off : l - (double)(k0 + j) * invN + cN;
     if (logw_out) logw_out[j] = lw;
@@ -1200,7 +1496,7 @@ inline __device__ void evidence_add(EvidState& E, int N, int n, const float* __r
     return;
   }
   double sw = 0.0, swl = 0.0;
-  for (int j = tid; j < n; j += B) {
+  for (int j = first; j < n; j += B) {
     const double l = (double)l_in[j];
     const double lw = live ? l + live_off : l - (double)(k0 + j) * invN + cN;
     const double w = exp(lw - mx);

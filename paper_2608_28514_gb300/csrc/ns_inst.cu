@@ -12,18 +12,51 @@ namespace nsd {
 #define NS_CAT2(a, b) a##b
 #define NS_CAT(a, b) NS_CAT2(a, b)
 
-cudaError_t NS_CAT(launch_run_, NS_DMAX)(const RunDesc* runs, const int* ids, int n, int block, size_t smem,
-                                         int chunk, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_run<NS_DMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// Launches n runs as clusters of `cluster` blocks (blocks r*cluster ..
+// r*cluster + cluster - 1 are run r's).
+template <class K>
+static cudaError_t launch_runs(K* kernel, const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk,
+                               int vb, int cluster, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_run<NS_DMAX><<<n, block, smem, s>>>(runs, ids, chunk);
-  return cudaGetLastError();
+  if (cluster <= 1) {
+    kernel<<<n, block, smem, s>>>(runs, ids, chunk, vb);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n * cluster), 1, 1);
+  cfg.blockDim = dim3((unsigned)block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, runs, ids, chunk, vb);
 }
 
-cudaError_t NS_CAT(occupancy_run_, NS_DMAX)(int block, size_t smem, int* blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(k_run<NS_DMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// The thread-walker kernel exists for the register classes whose walker (x,
+// v and a candidate in registers) fits 128 registers; the wider classes
+// always walk in groups.
+constexpr bool kHasThread = NS_DMAX <= kThreadWalkerMaxDim;
+
+cudaError_t NS_CAT(launch_run_, NS_DMAX)(const RunDesc* runs, const int* ids, int n, int block, size_t smem,
+                                         int chunk, int vb, int group, int cluster, cudaStream_t s) {
+  if constexpr (kHasThread)
+    if (!group) return launch_runs(k_run<NS_DMAX, kModeThread>, runs, ids, n, block, smem, chunk, vb, 1, s);
+  return launch_runs(k_run<NS_DMAX, kModeGroup>, runs, ids, n, block, smem, chunk, vb, cluster, s);
+}
+
+cudaError_t NS_CAT(occupancy_run_, NS_DMAX)(int block, size_t smem, int group, int* blocks_per_sm) {
+  auto* kernel = k_run<NS_DMAX, kModeGroup>;
+  if constexpr (kHasThread)
+    if (!group) kernel = k_run<NS_DMAX, kModeThread>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_run<NS_DMAX>, block, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, block, smem);
 }
 
 cudaError_t NS_CAT(launch_loglike_, NS_DMAX)(const LikParams& P, int n, const float* x, float* out,
@@ -44,9 +77,10 @@ cudaError_t NS_CAT(launch_slice_, NS_DMAX)(const LikParams& P, const SliceCfg& S
                                                       dir_scratch);
     return cudaGetLastError();
   }
-  k_slice<NS_DMAX><<<(m + 127) / 128, 128, sizeof(float) * 128 * dir_row(NS_DMAX), s>>>(P, SC, m, n_pad, correction, live_x, live_l, seed_slot, W, chol,
-                                                   cid, new_x, new_l, hist_l, hist_x, hist_len, evals, flags,
-                                                   dir_scratch);
+  k_slice<NS_DMAX><<<(m + kSliceWalkers - 1) / kSliceWalkers, kSliceThreads,
+                     sizeof(float) * kSliceWalkers * group_floats(NS_DMAX), s>>>(
+      P, SC, m, n_pad, correction, live_x, live_l, seed_slot, W, chol, cid, new_x, new_l, hist_l, hist_x, hist_len,
+      evals, flags, dir_scratch);
   return cudaGetLastError();
 }
 
@@ -56,25 +90,7 @@ cudaError_t NS_CAT(launch_slice_, NS_DMAX)(const LikParams& P, const SliceCfg& S
 // r*cluster + cluster - 1), which share its tensor-core evaluations.
 cudaError_t launch_run_mlp(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk, int cluster,
                            cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(k_run<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  if (cluster <= 1) {
-    k_run<32, true><<<n, block, smem, s>>>(runs, ids, chunk);
-    return cudaGetLastError();
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n * cluster), 1, 1);
-  cfg.blockDim = dim3((unsigned)block, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)cluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_run<32, true>, runs, ids, chunk);
+  return launch_runs(k_run<32, kModeMlp>, runs, ids, n, block, smem, chunk, block, cluster, s);
 }
 #endif
 

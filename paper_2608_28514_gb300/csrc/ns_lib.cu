@@ -100,7 +100,7 @@ __global__ void k_evidence(int N, int n, const float* __restrict__ l, double* st
     E.k = (long long)state[2];
   }
   __syncthreads();
-  evidence_add(E, N, n, l, logw, live != 0, S);
+  evidence_add(E, N, n, l, logw, live != 0, S, blockDim.x);
   if (threadIdx.x == 0) {
     state[0] = E.logz;
     state[1] = E.info;
@@ -112,7 +112,7 @@ __global__ void k_cluster(RunDesc R, uint32_t t) {
   extern __shared__ __align__(16) char sm[];
   __shared__ BlockScratch S;
   const Carve cv = make_carve(R.d, 1, R.n_nodes, kMaxDim, false, R.spill != 0);
-  cluster_phase(R, t, sm, cv, S);
+  cluster_phase(R, t, sm, cv, S, blockDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -143,12 +143,12 @@ void set_err(std::string* dst, const char* fmt, ...) {
 
 struct ClassFns {
   int dmax;
-  cudaError_t (*run)(const RunDesc*, const int*, int, int, size_t, int, cudaStream_t);
+  cudaError_t (*run)(const RunDesc*, const int*, int, int, size_t, int, int, int, int, cudaStream_t);
   cudaError_t (*ll)(const LikParams&, int, const float*, float*, cudaStream_t);
   cudaError_t (*sl)(const LikParams&, const SliceCfg&, int, int, int, const float*, const float*, const int*,
                     const float*, const float*, const int*, float*, float*, float*, float*, int*, long long*, int*,
                     float*, int, cudaStream_t);
-  cudaError_t (*occ)(int, size_t, int*);
+  cudaError_t (*occ)(int, size_t, int, int*);
 };
 #define NS_CLASS_ENTRY(D) {D, launch_run_##D, launch_loglike_##D, launch_slice_##D, occupancy_run_##D},
 const ClassFns kClasses[] = {NS_FOR_EACH_CLASS(NS_CLASS_ENTRY)};
@@ -232,6 +232,87 @@ int block_for_m(int m) {
   if (b < 128) b = 128;
   if (b > 256) b = 256;
   return b;
+}
+
+// How the analytic runs of each register class sit on the GPU (RunMode): the
+// block, whether the walkers are lane groups, and the blocks per run.
+//
+// A walk is a chain of dependent likelihoods, so lanes beyond one per walker
+// shorten it (slice_walker_lanes) as long as the SMs are not already full of
+// walkers.  Every class starts with the block that one walker per thread
+// needs; while the runs' threads stay within what the SMs hold at 128
+// registers (512 each), the class whose runs take longest gets twice the
+// lanes, first a wider block, then a cluster of blocks on as many SMs, up to
+// eight lanes per walker on blocks of 128 busy threads.  A batch that fills
+// the GPU by itself keeps one walker per thread, unless its blocks leave at
+// least four lanes per walker idle anyway.
+struct ClassNeed {
+  int dmax, n, max_m, n_steps;  // runs, largest batch and slice steps of a class
+};
+struct RunShape {
+  int block, vb, group, cluster, group_w;
+  double est;  // relative time of an iteration's walk
+};
+void shape_lanes(const ClassNeed& c, RunShape& q) {
+  q.group_w = (c.max_m + q.cluster - 1) / q.cluster;
+  const int G = group_lanes(q.block, q.group_w);
+  // rounds of likelihoods per slice step, and their cost
+  const double rounds = G >= 8 ? 2.3 : (G >= 4 ? 3.0 : (G >= 2 ? 4.5 : 7.0));
+  q.est = c.n_steps * rounds * (100.0 + 8.0 * c.dmax);
+}
+std::vector<RunShape> plan_shapes(const std::vector<ClassNeed>& need, int n_sm) {
+  std::vector<RunShape> out(need.size());
+  long long threads = 0;
+  for (size_t k = 0; k < need.size(); ++k) {
+    RunShape& q = out[k];
+    q.vb = q.block = block_for_m(need[k].max_m);
+    q.cluster = 1;
+    if (need[k].dmax > kThreadWalkerMaxDim) {  // no thread walkers: two lanes each at least
+      if (2 * need[k].max_m > q.block) q.block = 256;
+      if (2 * need[k].max_m > q.block) q.cluster = 2;
+    }
+    shape_lanes(need[k], q);
+    threads += (long long)need[k].n * q.block * q.cluster;
+  }
+  const long long budget = 512LL * n_sm;
+  const bool roomy = threads <= budget / 2;
+  std::vector<char> settled(need.size(), 0);
+  for (;;) {
+    int best = -1;
+    for (size_t k = 0; k < need.size(); ++k)
+      if (!settled[k] && (best < 0 || out[k].est > out[best].est)) best = (int)k;
+    if (best < 0) break;
+    const ClassNeed& c = need[best];
+    RunShape q = out[best];
+    if (q.block < 256 && 8 * q.group_w > q.block) q.block = 256;
+    else if (q.cluster < kGroupClusterMax && 128 * q.cluster < 8 * c.max_m) q.cluster *= 2;
+    else settled[best] = 1;
+    const long long more = (long long)c.n * (q.block * q.cluster - out[best].block * out[best].cluster);
+    if (threads + more > budget) settled[best] = 1;
+    if (settled[best]) continue;
+    threads += more;
+    shape_lanes(c, q);
+    out[best] = q;
+  }
+  for (size_t k = 0; k < need.size(); ++k) {
+    RunShape& q = out[k];
+    const int G = group_lanes(q.block, q.group_w);
+    q.group = need[k].dmax > kThreadWalkerMaxDim || G >= (roomy ? 2 : 4);
+    if (!q.group) {
+      q.block = q.vb;
+      q.cluster = 1;
+      q.group_w = 0;
+    }
+  }
+  return out;
+}
+
+int device_sms() {
+  int dev = 0, n_sm = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    n_sm = 1;
+  return n_sm;
 }
 
 bool finite_pos(double v) { return std::isfinite(v) && v > 0; }
@@ -456,7 +537,10 @@ struct HostRun {
 
 struct ClassGroup {
   int dmax = 0, block = 0, n = 0;
-  int cluster = 1;  // MLP group: CTAs per run
+  int cluster = 1;  // CTAs per run
+  int vb = 0;       // analytic runs: threads whose order the sums follow (RunShape)
+  int group = 0;    // analytic runs: walkers are lane groups
+  double est = 1e30;  // relative time of an iteration (MLP runs: the longest)
   bool mlp = false;
   size_t smem = 0;
   int* d_ids = nullptr;
@@ -464,7 +548,7 @@ struct ClassGroup {
 
 cudaError_t launch_class(const ClassGroup& g, const RunDesc* d_runs, int chunk, cudaStream_t s) {
   if (g.mlp) return launch_run_mlp(d_runs, g.d_ids, g.n, g.block, g.smem, chunk, g.cluster, s);
-  return kClasses[class_index(g.dmax)].run(d_runs, g.d_ids, g.n, g.block, g.smem, chunk, s);
+  return kClasses[class_index(g.dmax)].run(d_runs, g.d_ids, g.n, g.block, g.smem, chunk, g.vb, g.group, g.cluster, s);
 }
 
 }  // namespace
@@ -788,6 +872,24 @@ ns_status ns_create_batch(int n_runs, const ns_problem* runs, const ns_options* 
     set_err(nullptr, "device setup failed: %s", cudaGetErrorString(e));
     return fail(NS_ERR_CUDA);
   }
+  const int n_sm = device_sms();
+  std::vector<RunShape> shapes(kNumClasses + 1);
+  {
+    std::vector<ClassNeed> need;
+    std::vector<int> which;
+    for (int ci = 0; ci < kNumClasses; ++ci) {
+      if (counts[ci] == 0) continue;
+      ClassNeed c = {kClasses[ci].dmax, counts[ci], 1, 1};
+      for (int r : members[ci]) {
+        c.max_m = std::max(c.max_m, runs[r].m);
+        c.n_steps = std::max(c.n_steps, runs[r].n_slice_steps);
+      }
+      need.push_back(c);
+      which.push_back(ci);
+    }
+    const std::vector<RunShape> q = plan_shapes(need, n_sm);
+    for (size_t k = 0; k < q.size(); ++k) shapes[which[k]] = q[k];
+  }
   for (int ci = 0; ci <= kNumClasses; ++ci) {
     if (counts[ci] == 0) continue;
     ClassGroup g;
@@ -797,11 +899,21 @@ ns_status ns_create_batch(int n_runs, const ns_problem* runs, const ns_options* 
     g.d_ids = reinterpret_cast<int*>(base + off_ids[ci]);
     int maxm = 1;
     size_t smem = 0;
-    for (int r : members[ci]) {
-      maxm = std::max(maxm, runs[r].m);
-      smem = std::max(smem, make_carve(runs[r].d, runs[r].m, n_nodes, g.dmax, g.mlp, off[r].spill != 0).total);
+    for (int r : members[ci]) maxm = std::max(maxm, runs[r].m);
+    if (g.mlp) {
+      g.block = block_for_m(maxm);
+    } else {
+      const RunShape& q = shapes[ci];
+      g.est = q.est;
+      g.block = q.block;
+      g.vb = q.vb;
+      g.group = q.group;
+      g.cluster = q.cluster;
     }
-    g.block = block_for_m(maxm);
+    for (int r : members[ci])
+      smem = std::max(smem, make_carve(runs[r].d, runs[r].m, n_nodes, g.dmax, g.mlp, off[r].spill != 0,
+                                       g.group ? (runs[r].m + g.cluster - 1) / g.cluster : 0)
+                                .total);
     if (g.mlp) {
       g.block = std::max(g.block, kMlpThreads);  // the BF16 evaluator's warp roles
       // FP32 on the tensor cores needs BF16-valued weights; CTAs per run
@@ -818,10 +930,6 @@ ns_status ns_create_batch(int n_runs, const ns_problem* runs, const ns_options* 
         fits2 = fits2 && mlp_cluster_fits(M, 2);
         fits4 = fits4 && mlp_cluster_fits(M, 4);
       }
-      int dev = 0, n_sm = 1;
-      if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) !=
-                                                   cudaSuccess)
-        n_sm = 1;
       if (opt.mlp_cluster == 0) {
         g.cluster = (fits4 && 4 * g.n <= n_sm) ? 4 : ((fits2 && 2 * g.n <= n_sm) ? 2 : 1);
       } else {
@@ -847,6 +955,9 @@ ns_status ns_create_batch(int n_runs, const ns_problem* runs, const ns_options* 
     }
     h->groups.push_back(g);
   }
+  // the classes that take longest are launched first
+  std::stable_sort(h->groups.begin(), h->groups.end(),
+                   [](const ClassGroup& a, const ClassGroup& b) { return a.est > b.est; });
   if (h->groups.size() > 1) {
     e = cudaEventCreateWithFlags(&h->gfork, cudaEventDisableTiming);
     for (size_t gi = 0; gi < h->groups.size() && e == cudaSuccess; ++gi) {
@@ -891,13 +1002,15 @@ int ns_resident_runs_per_sm(int d, int m, int depth) {
   const int n_nodes = (1 << (depth + 1)) - 1;
   const int ci = class_index(d);
   int blocks = 0;
-  const cudaError_t e =
-      kClasses[ci].occ(block_for_m(m), make_carve(d, m, n_nodes, kClasses[ci].dmax).total, &blocks);
+  // the shape of a batch of many runs
+  const RunShape q = plan_shapes({{kClasses[ci].dmax, 1 << 20, m, 5 * d}}, device_sms())[0];
+  const cudaError_t e = kClasses[ci].occ(
+      q.block, make_carve(d, m, n_nodes, kClasses[ci].dmax, false, false, q.group_w).total, q.group, &blocks);
   if (e != cudaSuccess) {
     set_err(nullptr, "occupancy query failed: %s", cudaGetErrorString(e));
     return -1;
   }
-  return blocks;
+  return std::max(1, blocks / q.cluster);
 }
 
 ns_status ns_reset(ns_handle* h, void* stream) {
@@ -1575,14 +1688,15 @@ ns_status ns_run_noalloc(const ns_problem* problem, const ns_options* opt_in, fl
   NS_CUDA(cudaMemsetAsync(base + o_state, 0, sizeof(RunState), s), nullptr);
   const RunDesc* d_desc = reinterpret_cast<const RunDesc*>(base + o_desc);
   const int* d_ids = reinterpret_cast<const int*>(base + o_ids);
-  const int block = block_for_m(m);
-  const size_t smem = make_carve(d, m, n_nodes, dmax_class(d), false, spill).total;
+  const RunShape q = plan_shapes({{dmax_class(d), 1, m, p.n_slice_steps}}, device_sms())[0];
+  const size_t smem = make_carve(d, m, n_nodes, dmax_class(d), false, spill, q.group_w).total;
   const int chunk = opt.chunk_iters > 0 ? opt.chunk_iters : 1000;
   const long long max_rounds = opt.max_iter / chunk + 2;
   RunState hs;
   std::memset(&hs, 0, sizeof(hs));
   for (long long round = 0;; ++round) {
-    const cudaError_t e = kClasses[class_index(d)].run(d_desc, d_ids, 1, block, smem, chunk, s);
+    const cudaError_t e =
+        kClasses[class_index(d)].run(d_desc, d_ids, 1, q.block, smem, chunk, q.vb, q.group, q.cluster, s);
     NS_CUDA(e, nullptr);
     NS_CUDA(cudaMemcpyAsync(&hs, base + o_state, sizeof(RunState), cudaMemcpyDeviceToHost, s), nullptr);
     NS_CUDA(cudaStreamSynchronize(s), nullptr);

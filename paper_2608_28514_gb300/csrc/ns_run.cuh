@@ -103,8 +103,10 @@ __host__ __device__ constexpr int mlp_xs(int d) { return (d + 3) & ~3; }
 // spill: the run's cluster tables do not fit next to the rest (large d or a
 // deep tree); the Cholesky factors and the tree scratch then stay in global
 // memory (only the clustering and the direction draws read them).
+// group_w: walkers of one block when a walker is a group of lanes
+// (slice_walker_lanes), 0 when it is a thread.
 __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax, bool mlp = false,
-                                            bool spill = false) {
+                                            bool spill = false, int group_w = 0) {
   Carve c;
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -151,7 +153,8 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
   if (!mlp) {
     const size_t end_cluster = o;
     o = phase0;
-    c.slots = take(sizeof(float) * (size_t)dir_row(dmax) * (m + 31) / 32 * 32);
+    c.slots = take(group_w > 0 ? sizeof(float) * (size_t)group_floats(dmax) * group_w
+                               : sizeof(float) * (size_t)dir_row(dmax) * (m + 31) / 32 * 32);
     const size_t end_slots = o;
     o = phase0;
     c.candA = take(cand_bytes);
@@ -209,7 +212,7 @@ inline __device__ void init_live(const RunDesc& R, const LikParams& P) {
 // a3 (section 2.1): the root node is the whole live set (mean, covariance,
 // regularised FP64 Cholesky); for depth >= 1 the tree of cluster_tree
 // follows.
-inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, const Carve& cv, BlockScratch& S) {
+inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, const Carve& cv, BlockScratch& S, int vb) {
   const int d = R.d;
   float* tile = reinterpret_cast<float*>(sm + cv.tile);
   double* acc = reinterpret_cast<double*>(sm + cv.acc);
@@ -295,6 +298,7 @@ inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, con
   io.s_cent = s_cent;
   io.s_mask = s_mask;
   io.bracket = R.bracket;
+  io.vb = vb;
   cluster_tree(io, T, S, nw_chol);
 }
 
@@ -348,19 +352,20 @@ __device__ __noinline__ void walker_phase(const RunDesc& R, const LikParams& P, 
 }
 
 // a4-a7 with one walker per warp (RunDesc::walker_warp): warp w takes the
-// walkers w, w + n_warps, ... in turn.  On return lane 0 of each warp holds
+// walkers w0 + w, w0 + w + n_warps, ... below w1 in turn.  On return lane 0 of each warp holds
 // in ev its walkers' likelihood evaluations and in fl how many of them hit a
 // step-out or shrink cap (other lanes 0).  Called by every thread.
 template <int DMAX>
 __device__ __noinline__ void walker_phase_warp(const RunDesc& R, const LikParams& P, const SliceCfg& SC,
-                                               const float* s_W, const int* s_seed, long long& ev, int& fl) {
+                                               const float* s_W, const int* s_seed, int w0, int w1, long long& ev,
+                                               int& fl) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, m = R.m, d = R.d;
   LaneLik<DMAX> Q;
   lane_lik<DMAX>(P, Q);
   const float thr_out = (R.correction == 3) ? s_W[m - 1] : s_W[0];
   long long e_sum = 0;
   int n_cap = 0;
-  for (int i = wid; i < m; i += nw) {
+  for (int i = w0 + wid; i < w1; i += nw) {
     const int sd = s_seed[i];
     const float thr_in = (R.correction == 3) ? s_W[m - 1] : s_W[i];
     WalkerOut O;
@@ -382,6 +387,120 @@ __device__ __noinline__ void walker_phase_warp(const RunDesc& R, const LikParams
   }
   ev = (lane == 0) ? e_sum : 0;
   fl = (lane == 0) ? n_cap : 0;
+}
+
+// Lanes of each of W walkers' groups in a block of B >= W threads: the
+// largest power of two that fits, at most 8 (four candidates on each side of
+// the stepping out; more would seldom be used).
+__host__ __device__ inline int group_lanes(int B, int W) {
+  int G = 1;
+  while (G < 8 && 2 * G * W <= B) G *= 2;
+  return G;
+}
+
+// a4-a7 of the walkers [w0, w1) on the calling block, a group of lanes each
+// (or, with RunDesc::walker_warp, a warp each in turn): the direction rows,
+// spread over the block, then the walks.  mem: group_floats(DMAX) floats of
+// shared memory per walker; s_off: int [m] of shared memory.  On return each
+// walker's first lane holds its evaluations in ev and 1 in fl if it hit a
+// cap (walker_warp: lane 0 of each warp its walkers' sums).  Every thread of
+// the block; live_l, live_x and live_cid may have been written by another
+// SM of the cluster before its last barrier.
+template <int DMAX>
+__device__ __noinline__ void group_phase(const RunDesc& R, const LikParams& P, const SliceCfg& SC, int w0, int w1,
+                                         const float* s_W, const int* s_seed, const float* s_chol, int* s_off,
+                                         float* mem, long long& ev, int& fl, long long& cyc_draw,
+                                         long long& cyc_walk) {
+  const int tid = threadIdx.x, m = R.m, d = R.d;
+  const long long c0 = clock64();
+  for (int w = w0 + tid; w < w1; w += blockDim.x) s_off[w] = R.live_cid[s_seed[w]] * d * d;
+  __syncthreads();
+  draw_directions_block<DMAX>(SC, w0, w1, [&](int w) { return s_chol + s_off[w]; }, R.dirs);
+  const long long c1 = clock64();
+  ev = 0;
+  fl = 0;
+  if (R.walker_warp) {
+    walker_phase_warp<DMAX>(R, P, SC, s_W, s_seed, w0, w1, ev, fl);
+  } else {
+    const int G = group_lanes(blockDim.x, w1 - w0);
+    if (w0 + (tid & ~31) / G < w1) {  // warps that hold a walker
+      const bool act = w0 + tid / G < w1;
+      const int i = act ? w0 + tid / G : w0;
+      const int sd = s_seed[i];
+      const float thr_out = (R.correction == 3) ? s_W[m - 1] : s_W[0];
+      const float thr_in = (R.correction == 3) ? s_W[m - 1] : s_W[i];
+      WalkerOut O;
+      O.new_x = R.new_x + (size_t)i * d;
+      O.new_l = R.new_l + i;
+      O.hist_l = R.hist_l + (size_t)i * R.t_max;
+      O.hist_x = R.hist_x + (size_t)i * R.t_max * d;
+      O.hist_len = R.hist_len + i;
+      slice_walker_any<DMAX>(P, SC, G, i, act, R.live_x + sd, R.n_pad, R.live_l[sd],
+                             R.dirs + (size_t)i * SC.n_steps * dir_row(DMAX),
+                             mem + (size_t)(i - w0) * group_floats(DMAX), thr_out, thr_in, O, ev, fl);
+      if (act && tid % G == 0 && R.wk_evals) {
+        R.wk_evals[i] = (int)ev;
+        R.wk_flags[i] = fl;
+      }
+      fl = fl ? 1 : 0;
+    }
+  }
+  cyc_draw = c1 - c0;
+  cyc_walk = clock64() - c1;
+}
+
+// CTA 0's mailbox of an analytic run that is spread over a cluster of C
+// CTAs (same address in every CTA): the command of the iteration, and each
+// follower's evaluation and cap counts.
+constexpr int kGroupClusterMax = 8;
+struct GroupMail {
+  int op;        // 0 exit, 1 walk, 2 reload the cluster factors, then walk
+  uint32_t t;
+  int ev[kGroupClusterMax], fl[kGroupClusterMax];
+};
+
+// The walkers of CTA `rank` of C.
+__device__ __forceinline__ int group_share(int m, unsigned C, unsigned rank) { return (int)((unsigned)m * rank / C); }
+
+// A follower CTA: walks its share of every iteration's walkers until CTA 0
+// posts the exit.  CTA 0's selection (W and the start slots) is read from
+// its shared memory; the live set and the cluster factors from global
+// memory; the new points go back through global memory.  The cluster
+// barriers order all of it.
+template <int DMAX>
+__device__ void group_follower(const RunDesc& R, const LikParams& P, SliceCfg SC, char* sm, const Carve& cv,
+                               BlockScratch& S, GroupMail* mail, unsigned C, unsigned rank) {
+  const int tid = threadIdx.x, B = blockDim.x, m = R.m, d = R.d;
+  const int w0 = group_share(m, C, rank), w1 = group_share(m, C, rank + 1);
+  float* s_chol = cv.chol_global ? R.chol : reinterpret_cast<float*>(sm + cv.chol);
+  float* s_W = reinterpret_cast<float*>(sm + cv.W);
+  int* s_seed = reinterpret_cast<int*>(sm + cv.seed);
+  int* s_off = reinterpret_cast<int*>(sm + cv.stage_cid);
+  float* mem = reinterpret_cast<float*>(sm + cv.slots);
+  const unsigned mail0 = cl_map(smem_u32(mail), 0), W0 = cl_map(smem_u32(s_W), 0), seed0 = cl_map(smem_u32(s_seed), 0);
+  for (;;) {
+    cl_sync();  // the command is posted
+    const int op = cl_ld_s32(mail0 + (unsigned)offsetof(GroupMail, op));
+    if (op == 0) break;
+    SC.t = (uint32_t)cl_ld_s32(mail0 + (unsigned)offsetof(GroupMail, t));
+    for (int i = tid; i < m; i += B) {
+      s_W[i] = cl_ld_f32(W0 + 4u * i);
+      s_seed[i] = cl_ld_s32(seed0 + 4u * i);
+    }
+    if (op == 2 && !cv.chol_global)
+      for (int i = tid; i < R.n_nodes * d * d; i += B) s_chol[i] = R.chol[i];
+    __syncthreads();
+    long long ev = 0, c0 = 0, c1 = 0;
+    int fl = 0;
+    group_phase<DMAX>(R, P, SC, w0, w1, s_W, s_seed, s_chol, s_off, mem, ev, fl, c0, c1);
+    const int evs = (int)block_sum_ll(ev, S), fls = (int)block_sum_ll(fl, S);
+    if (tid == 0) {
+      cl_st_s32(mail0 + (unsigned)offsetof(GroupMail, ev) + 4u * rank, evs);
+      cl_st_s32(mail0 + (unsigned)offsetof(GroupMail, fl) + 4u * rank, fls);
+    }
+    cl_sync();  // the new points and the counts are in place
+  }
+  cl_sync();  // CTA 0's mailbox has been read
 }
 
 // a4-a7 for MLP runs: the walkers advance in lock step, one round at a time;
@@ -992,24 +1111,31 @@ inline __device__ void init_live_mlp(const RunDesc& R, float* xbuf, float* lbuf,
   }
 }
 
-// Blocks of up to 256 threads.  For the small register classes two such
-// blocks per SM cap the registers at 128 per thread (more runs resident per
-// SM hide the walkers' latency); the wide classes keep the full register
-// file.  NS_RUN_MINB overrides the choice at build time.
+// How a run's walkers sit on its block: one per thread (the small register
+// classes, when the runs fill the GPU), the lock-step rounds of an MLP run,
+// or a group of lanes each (and, with few runs, a cluster of blocks per run).
+enum RunMode { kModeThread = 0, kModeMlp = 1, kModeGroup = 2 };
+constexpr int kThreadWalkerMaxDim = 12;  // widest register class with a thread-walker kernel
+
+// Blocks of up to 256 threads, 128 registers per thread (two such blocks,
+// or four of 128 threads, per SM).  NS_RUN_MINB and NS_RUN_MAXNREG (build
+// time) override the cap of the thread-walker kernels.
 #ifdef NS_RUN_MINB
-#define NS_MINB(D) NS_RUN_MINB
+#define NS_MINB(MODE) ((MODE) == kModeThread ? NS_RUN_MINB : 2)
 #else
-#define NS_MINB(D) ((D) <= 12 ? 2 : 1)
+#define NS_MINB(MODE) 2
 #endif
-// NS_RUN_MAXNREG (build time) caps the analytic run kernels' registers per
-// thread directly instead (finer than whole blocks per SM).
 #ifdef NS_RUN_MAXNREG
-#define NS_RUN_BOUNDS(MLP, D) __launch_bounds__((MLP ? kMlpThreads : 256)) __maxnreg__(MLP ? 200 : NS_RUN_MAXNREG)
+#define NS_RUN_BOUNDS(MODE)                                \
+  __launch_bounds__(((MODE) == kModeMlp ? kMlpThreads : 256)) \
+      __maxnreg__((MODE) == kModeMlp ? 200 : ((MODE) == kModeThread ? NS_RUN_MAXNREG : 128))
 #else
-#define NS_RUN_BOUNDS(MLP, D) __launch_bounds__((MLP ? kMlpThreads : 256), (MLP ? 1 : NS_MINB(D)))
+#define NS_RUN_BOUNDS(MODE) \
+  __launch_bounds__(((MODE) == kModeMlp ? kMlpThreads : 256), ((MODE) == kModeMlp ? 1 : NS_MINB(MODE)))
 #endif
-template <int DMAX, bool MLP = false>
-__global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs, const int* __restrict__ ids, int chunk) {
+template <int DMAX, int MODE>
+__global__ void NS_RUN_BOUNDS(MODE) k_run(const RunDesc* __restrict__ runs, const int* __restrict__ ids, int chunk, int vb) {
+  constexpr bool MLP = MODE == kModeMlp;
   extern __shared__ __align__(16) char sm[];
   __shared__ RunDesc R;
   __shared__ RunState RS;
@@ -1018,9 +1144,17 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
   __shared__ MlpCtx mlp_ctx;
   const int tid = threadIdx.x, B = blockDim.x;
   // MLP runs may be launched as clusters of C CTAs per run (CTA 0 runs the
-  // sampler, the others share its tensor-core evaluations)
+  // sampler, the others share its tensor-core evaluations), group-walker
+  // runs too (the others take a share of the walkers)
   unsigned C = 1, rank = 0;
   ClusterMail* mail = nullptr;
+  GroupMail* gmail = nullptr;
+  if constexpr (MODE == kModeGroup) {
+    __shared__ GroupMail g_mail;
+    gmail = &g_mail;
+    C = cl_size();
+    rank = cl_rank();
+  }
   if constexpr (MLP) {
     __shared__ ClusterMail cl_mail;
     mail = &cl_mail;
@@ -1036,7 +1170,8 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
   }
   __syncthreads();
   const int d = R.d, N = R.N, m = R.m;
-  const Carve cv = make_carve(d, m, R.n_nodes, DMAX, MLP, R.spill != 0);
+  const Carve cv = make_carve(d, m, R.n_nodes, DMAX, MLP, R.spill != 0,
+                              MODE == kModeGroup ? (m + (int)C - 1) / (int)C : 0);
   if constexpr (MLP) {
     if (rank > 0) {
       mlp_follower(R, &mlp_ctx, mail, align1024_shared(sm + cv.mlp), C, rank);
@@ -1047,7 +1182,7 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
     if constexpr (MLP) {
       if (C > 1) mlp_leader_exit(&mlp_ctx, mail, false);
     }
-    return;
+    return;  // (group-walker clusters: every CTA reads the same state)
   }
   if constexpr (MLP) {
     if (R.precision != 0) mlp_ctx_init(&mlp_ctx);
@@ -1081,6 +1216,24 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
     int* dst = reinterpret_cast<int*>(&P);
     for (int i = tid; i < (int)(sizeof(LikParams) / 4); i += B) dst[i] = src[i];
   }
+  SliceCfg SC;
+  SC.d = d;
+  SC.n_steps = R.n_steps;
+  SC.e_max = R.e_max;
+  SC.s_max = R.s_max;
+  SC.t_max = R.t_max;
+  SC.width = R.width;
+  SC.k0 = R.k0;
+  SC.k1 = R.k1;
+  if constexpr (MODE == kModeGroup) {
+    if (rank > 0) {  // the factors of the last re-clustering, then CTA 0's commands
+      if (RS.t > 0 && !cv.chol_global)
+        for (int i = tid; i < R.n_nodes * d * d; i += B) s_chol[i] = R.chol[i];
+      __syncthreads();
+      group_follower<DMAX>(R, P, SC, sm, cv, S, gmail, C, rank);
+      return;
+    }
+  }
   __syncthreads();
   if (!RS.initialized) {
     if constexpr (MLP) init_live_mlp<DMAX>(R, s_xbuf, s_lbuf, s_rlist, s_mlp);
@@ -1103,15 +1256,6 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
   __syncthreads();
 
   const double Nd = (double)N;
-  SliceCfg SC;
-  SC.d = d;
-  SC.n_steps = R.n_steps;
-  SC.e_max = R.e_max;
-  SC.s_max = R.s_max;
-  SC.t_max = R.t_max;
-  SC.width = R.width;
-  SC.k0 = R.k0;
-  SC.k1 = R.k1;
 
   for (int it = 0; it < chunk; ++it) {
     if (RS.stopped || RS.status != 0) break;
@@ -1130,7 +1274,8 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
       }
     };
     // a3: clustering
-    if (R.recluster_every > 0 && (t % (uint32_t)R.recluster_every) == 0) cluster_phase(R, t, sm, cv, S);
+    const bool reclustered = R.recluster_every > 0 && (t % (uint32_t)R.recluster_every) == 0;
+    if (reclustered) cluster_phase(R, t, sm, cv, S, vb);
     tick(kPhCluster);
     // a1-a2: selection
     select_worst(R.live_l, N, m, R.k0, R.k1, t, s_sel_slot, s_sel_key, s_worst, s_W, s_seed, X, S);
@@ -1142,6 +1287,27 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
     if constexpr (MLP) {
       walker_phase_mlp<DMAX>(R, SC, s_W, s_seed, s_chol, s_xbuf, s_lbuf, s_rlist, s_mlp, &mlp_ctx, mail, s_list, S, ev,
                              fl, re, werr, cyc_eval, cyc_reeval, RS.mlp_count);
+    } else if constexpr (MODE == kModeGroup) {
+      if (C > 1) {
+        if (tid == 0) {
+          gmail->op = reclustered ? 2 : 1;
+          gmail->t = t;
+        }
+        cl_sync();
+      }
+      group_phase<DMAX>(R, P, SC, 0, group_share(m, C, 1), s_W, s_seed, s_chol, s_stage_cid, s_slots, ev, fl, cyc_eval,
+                        cyc_reeval);
+      if (C > 1) {
+        cl_sync();
+        if (tid > 0 && tid < (int)C) {
+          ev += gmail->ev[tid];
+          fl += gmail->fl[tid];
+        }
+      }
+      if (tid == 0) {
+        RS.cycles[6] += cyc_eval;
+        RS.cycles[7] += cyc_reeval;
+      }
     } else {
       // every walker's rows of the iteration, spread over the whole block;
       // the walkers' cluster-factor offsets first (the update phase's
@@ -1152,7 +1318,7 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
       draw_directions_block<DMAX>(SC, 0, m, [&](int w) { return s_chol + s_stage_cid[w]; }, R.dirs);
       const long long cd1 = clock64();
       if (R.walker_warp) {
-        walker_phase_warp<DMAX>(R, P, SC, s_W, s_seed, ev, fl);
+        walker_phase_warp<DMAX>(R, P, SC, s_W, s_seed, 0, m, ev, fl);
         cyc_reeval = clock64() - cd1;
       } else if ((tid & ~31) < m) {
         walker_phase<DMAX>(R, P, SC, s_W, s_seed, s_chol, s_slots, ev, fl, cyc_eval, cyc_reeval);
@@ -1241,7 +1407,7 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
     __syncthreads();
     tick(kPhUpdate);
     // a11: evidence (FP64)
-    evidence_add(E, N, m, A.l, R.dead_logw + nd0, false, S);
+    evidence_add(E, N, m, A.l, R.dead_logw + nd0, false, S, vb);
     float lm = -CUDART_INF_F;
     for (int j = tid; j < N; j += B) lm = fmaxf(lm, R.live_l[j]);
     const float lmax = block_max_f(lm, S);
@@ -1260,7 +1426,7 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
     if (flag_any) {
       // final live tail, slot order: each point carries X_K / N
       const long long nd1 = RS.n_dead;
-      evidence_add(E, N, N, R.live_l, R.dead_logw + nd1, true, S);
+      evidence_add(E, N, N, R.live_l, R.dead_logw + nd1, true, S, vb);
       for (int q = tid; q < N * d; q += B) {
         const int j = q / d, i = q - j * d;
         R.dead_x[(size_t)(nd1 + j) * d + i] = R.live_x[(size_t)i * R.n_pad + j];
@@ -1277,6 +1443,13 @@ __global__ void NS_RUN_BOUNDS(MLP, DMAX) k_run(const RunDesc* __restrict__ runs,
     }
   }
   __syncthreads();
+  if constexpr (MODE == kModeGroup) {
+    if (C > 1) {
+      if (tid == 0) gmail->op = 0;
+      cl_sync();
+      cl_sync();
+    }
+  }
   if constexpr (MLP) {
     if (C > 1) mlp_leader_exit(&mlp_ctx, mail, R.precision != 0);
     if (R.precision != 0) mlp_ctx_free(&mlp_ctx);
@@ -1299,20 +1472,25 @@ __global__ void k_loglike(const LikParams P, int n, const float* __restrict__ x,
   out[j] = loglike_u<DMAX>(P, xr);
 }
 
-// Step-level slice kernel: dir_scratch holds the walkers' per-step tables,
-// [m][n_steps][dir_row(DMAX)].
+// Step-level slice kernel: kSliceWalkers walkers per block, a group of
+// kSliceLanes lanes each (the rest of the block shares the direction draws).
+// dir_scratch holds the walkers' per-step tables, [m][n_steps][dir_row(DMAX)].
+// One call has at most 256 walkers, so blocks are kept small to put the
+// walks on as many SMs as there are (four walkers each: 64 blocks at m = 256).
+constexpr int kSliceWalkers = 4, kSliceLanes = 8, kSliceThreads = 128;
 template <int DMAX>
-__global__ void k_slice(const LikParams P, SliceCfg SC, int m, int n_pad, int correction,
-                        const float* __restrict__ live_x, const float* __restrict__ live_l,
-                        const int* __restrict__ seed_slot, const float* __restrict__ W,
-                        const float* __restrict__ chol, const int* __restrict__ cid, float* new_x,
-                        float* new_l, float* hist_l, float* hist_x, int* hist_len, long long* evals,
-                        int* flags, float* dir_scratch) {
+__global__ void __launch_bounds__(kSliceThreads)
+    k_slice(const LikParams P, SliceCfg SC, int m, int n_pad, int correction, const float* __restrict__ live_x,
+            const float* __restrict__ live_l, const int* __restrict__ seed_slot, const float* __restrict__ W,
+            const float* __restrict__ chol, const int* __restrict__ cid, float* new_x, float* new_l, float* hist_l,
+            float* hist_x, int* hist_len, long long* evals, int* flags, float* dir_scratch) {
   extern __shared__ __align__(16) char sm[];
-  const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const bool act = i0 < m;
-  const int i = act ? i0 : 0;
-  const int d = SC.d;
+  const int d = SC.d, w0 = blockIdx.x * kSliceWalkers, w1 = min(m, w0 + kSliceWalkers);
+  draw_directions_block<DMAX>(SC, w0, w1, [&](int w) { return chol + (size_t)cid[seed_slot[w]] * d * d; }, dir_scratch);
+  const int q = threadIdx.x / kSliceLanes;
+  if ((int)(threadIdx.x & ~31u) / kSliceLanes >= w1 - w0) return;  // warps without a walker
+  const bool act = w0 + q < w1;
+  const int i = act ? w0 + q : w0;
   const int sd = seed_slot[i];
   const float thr_out = (correction == 3) ? W[m - 1] : W[0];
   const float thr_in = (correction == 3) ? W[m - 1] : W[i];
@@ -1322,18 +1500,13 @@ __global__ void k_slice(const LikParams P, SliceCfg SC, int m, int n_pad, int co
   O.hist_l = hist_l + (size_t)i * SC.t_max;
   O.hist_x = hist_x + (size_t)i * SC.t_max * d;
   O.hist_len = hist_len + i;
-  float* my_dirs = dir_scratch + (size_t)i * SC.n_steps * dir_row(DMAX);
-  {  // this block's walkers' rows, spread over the block
-    const int w0 = blockIdx.x * blockDim.x, w1 = min(m, w0 + (int)blockDim.x);
-    if (w0 < w1)
-      draw_directions_block<DMAX>(SC, w0, w1, [&](int w) { return chol + (size_t)cid[seed_slot[w]] * d * d; },
-                                  dir_scratch);
-  }
   long long ev = 0;
   int fl = 0;
-  float* slot = reinterpret_cast<float*>(sm) + (size_t)threadIdx.x * dir_row(DMAX);
-  slice_walker<DMAX>(P, SC, i, act, live_x + sd, n_pad, live_l[sd], my_dirs, slot, thr_out, thr_in, O, ev, fl);
-  if (act) {
+  slice_walker_any<DMAX>(P, SC, kSliceLanes, i, act, live_x + sd, n_pad, live_l[sd],
+                           dir_scratch + (size_t)i * SC.n_steps * dir_row(DMAX),
+                           reinterpret_cast<float*>(sm) + (size_t)(i - w0) * group_floats(DMAX), thr_out, thr_in, O, ev,
+                           fl);
+  if (act && threadIdx.x % kSliceLanes == 0) {
     evals[i] = ev;
     flags[i] = fl;
   }
@@ -1382,14 +1555,14 @@ __global__ void k_slice_warp(const LikParams P, SliceCfg SC, int m, int n_pad, i
 // Launchers, one set per class (defined in ns_inst.cu).
 #define NS_DECLARE_LAUNCHERS(D)                                                                          \
   cudaError_t launch_run_##D(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk, \
-                             cudaStream_t s);                                                            \
+                             int vb, int group, int cluster, cudaStream_t s);                                                            \
   cudaError_t launch_loglike_##D(const LikParams& P, int n, const float* x, float* out, cudaStream_t s);  \
   cudaError_t launch_slice_##D(const LikParams& P, const SliceCfg& SC, int m, int n_pad, int correction,   \
                                const float* live_x, const float* live_l, const int* seed_slot,           \
                                const float* W, const float* chol, const int* cid, float* new_x,          \
                                float* new_l, float* hist_l, float* hist_x, int* hist_len, long long* evals, \
                                int* flags, float* dir_scratch, int warp, cudaStream_t s);                  \
-  cudaError_t occupancy_run_##D(int block, size_t smem, int* blocks_per_sm);
+  cudaError_t occupancy_run_##D(int block, size_t smem, int group, int* blocks_per_sm);
 NS_FOR_EACH_CLASS(NS_DECLARE_LAUNCHERS)
 cudaError_t launch_run_mlp(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk, int cluster,
                            cudaStream_t s);

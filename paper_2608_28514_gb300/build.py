@@ -1,7 +1,8 @@
 """Build the sm_103a shared library ``libns_gb300.so`` in-tree.
 
 The translation units compile in parallel (the host library and one
-instantiation of the per-dimension kernels for each register class), then
+instantiation of the per-dimension kernels for each register class, the wide
+ones in parts), then
 nvcc links them with the static CUDA runtime.  Objects go to ``_build/``.
 """
 import concurrent.futures as cf
@@ -21,9 +22,10 @@ CLASSES = (2, 4, 6, 8, 10, 12, 16, 20, 24, 28, 32)
 def _sources():
     out = [(os.path.join(CSRC, "ns_lib.cu"), os.path.join(BUILD, "ns_lib.o"), []),
            (os.path.join(CSRC, "ns_mlp.cu"), os.path.join(BUILD, "ns_mlp.o"), [])]
-    for d in CLASSES:
-        out.append((os.path.join(CSRC, "ns_inst.cu"), os.path.join(BUILD, f"ns_inst_{d}.o"),
-                    [f"-DNS_DMAX={d}"]))
+    for d in reversed(CLASSES):  # the longest first
+        for part in ((1, 2, 4) if d >= 16 else (7,)):
+            out.append((os.path.join(CSRC, "ns_inst.cu"), os.path.join(BUILD, f"ns_inst_{d}_{part}.o"),
+                        [f"-DNS_DMAX={d}", f"-DNS_PART={part}"]))
     return out
 
 
@@ -54,7 +56,7 @@ def build(force=False, verbose=False):
     os.makedirs(BUILD, exist_ok=True)
     nvcc = os.environ.get("NVCC", "nvcc")
     logs = []
-    workers = max(2, min(len(CLASSES) + 1, os.cpu_count() or 4))
+    workers = max(2, min(len(_sources()), os.cpu_count() or 4))
     with cf.ThreadPoolExecutor(max_workers=workers) as ex:
         futs = [ex.submit(_compile, s, o, e, nvcc, verbose) for s, o, e in _sources()]
         for f in futs:

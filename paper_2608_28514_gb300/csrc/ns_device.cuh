@@ -121,6 +121,9 @@ struct LikParams {
   float glw[kMaxGmmModes];         // log w_k
 };
 
+// The 32-bit shared-memory address of a pointer into shared memory.
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 
@@ -145,11 +148,11 @@ __device__ __forceinline__ bool candidate(const float (&x)[DMAX], const float (&
   return (mn >= 0.f) && (mx <= 1.f);
 }
 
-// logL at the unit-cube point u (zero beyond d) for one likelihood family.
-// Pairs of coordinates (and pairs of rows of L^T) go through one packed FMA
-// each.
+// logL at the unit-cube point u (zero beyond d) for one likelihood family,
+// NaN where it is not a number.  Pairs of coordinates (and pairs of rows of
+// L^T) go through one packed FMA each.
 template <int DMAX, int KIND>
-__device__ __forceinline__ float loglike_k(const LikParams& P, const float (&u)[DMAX]) {
+__device__ __forceinline__ float loglike_raw(const LikParams& P, const float (&u)[DMAX]) {
   float ll = -CUDART_INF_F;
   if constexpr (KIND == kIso) {
     float2 acc = f2(0.f, 0.f);
@@ -247,21 +250,32 @@ __device__ __forceinline__ float loglike_k(const LikParams& P, const float (&u)[
     const float z = sqrtf(acc.x + acc.y) - P.a;
     ll = -z * z * P.inv2s2;
   }
+  return ll;
+}
+
+// The same with -infinity for NaN.
+template <int DMAX, int KIND>
+__device__ __forceinline__ float loglike_k(const LikParams& P, const float (&u)[DMAX]) {
+  const float ll = loglike_raw<DMAX, KIND>(P, u);
   return (ll != ll) ? -CUDART_INF_F : ll;
 }
 
-// The same for a family known at run time.
+// The same for a family known at run time.  (One result at the end of the
+// switch: with a return in each case the families' tails are compiled apart,
+// and a 28-D mixture's walk took 20 % longer.)
 template <int DMAX>
 __device__ __forceinline__ float loglike_u(const LikParams& P, const float (&u)[DMAX]) {
+  float ll;
   switch (P.kind) {
-    case kIso: return loglike_k<DMAX, kIso>(P, u);
-    case kCorr: return loglike_k<DMAX, kCorr>(P, u);
-    case kRosen: return loglike_k<DMAX, kRosen>(P, u);
-    case kMix: return loglike_k<DMAX, kMix>(P, u);
-    case kGmm: return loglike_k<DMAX, kGmm>(P, u);
-    case kShell: return loglike_k<DMAX, kShell>(P, u);
-    default: return -CUDART_INF_F;
+    case kIso: ll = loglike_raw<DMAX, kIso>(P, u); break;
+    case kCorr: ll = loglike_raw<DMAX, kCorr>(P, u); break;
+    case kRosen: ll = loglike_raw<DMAX, kRosen>(P, u); break;
+    case kMix: ll = loglike_raw<DMAX, kMix>(P, u); break;
+    case kGmm: ll = loglike_raw<DMAX, kGmm>(P, u); break;
+    case kShell: ll = loglike_raw<DMAX, kShell>(P, u); break;
+    default: ll = -CUDART_INF_F;
   }
+  return (ll != ll) ? -CUDART_INF_F : ll;
 }
 
 // ---------------------------------------------------------------------------
@@ -689,7 +703,7 @@ inline __device__ void slice_walker(const LikParams& P, const SliceCfg& S, int w
   for (int j = 0; j < kPreShrink; ++j) pre[j] = 0.f;
   const bool was_active = active;
   int step = 0, phase = 0, nexp = 0, nsh = 0, hlen = 0, flags = 0;
-  long long evals = 0;
+  int evals = 0;
   float a = 0.f, b = 0.f;
   if (n_steps <= 0) active = false;
   if (active) {
@@ -1636,6 +1650,56 @@ inline __device__ void warp_eigen_clip(int d, const double* C, double delta, dou
   __syncwarp();
 }
 
+// Lanes that factorise one matrix: a lane per row, matrices side by side in a
+// warp.
+__host__ __device__ constexpr int chol_lanes(int dm) { return dm <= 4 ? 4 : (dm <= 8 ? 8 : (dm <= 16 ? 16 : 32)); }
+
+// The regularised Cholesky of section 2.1 with a lane per row, the row in
+// registers: lane i of each group of chol_lanes(DM) lanes holds row i of a
+// covariance in a[0..i] (lanes and entries beyond d: 0) and receives row i of
+// the factor of C + delta I, delta = 1e-10 tr(C) / d.  Right-looking: per
+// column one reciprocal square root of the pivot, then the trailing rows,
+// the other rows' column entries by shuffle (in shared memory each update
+// waited for the previous one's store).  reg = false: a is factorised as it
+// is.  Per group: 1 done (1e-6 I for a trace that is not positive), 0 a pivot
+// is not positive (a is then spoilt).
+template <int DM>
+__device__ __forceinline__ int reg_chol_rows(int d, int i, double (&a)[DM], bool reg = true) {
+  constexpr int GL = chol_lanes(DM);
+  double tr = 0.0;
+#pragma unroll
+  for (int k = 0; k < DM; ++k)
+    if (k == i) tr = a[k];
+#pragma unroll
+  for (int o = GL / 2; o > 0; o >>= 1) tr = __dadd_rn(tr, __shfl_xor_sync(kFull, tr, o, GL));
+  const bool fine = !reg || ((tr > 0.0) && isfinite(tr));
+  const double delta = 1e-10 * tr / d;
+#pragma unroll
+  for (int k = 0; k < DM; ++k)
+    if (reg && k == i && i < d) a[k] = __dadd_rn(a[k], delta);
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < DM; ++j)
+    if (j < d) {
+      const double s = __shfl_sync(kFull, a[j], j, GL);
+      ok = ok && (s > 0.0) && isfinite(s);
+      const double r = rsqrt(s);
+      const double lij = a[j] * r;
+      a[j] = i > j ? lij : (i == j ? s * r : a[j]);
+#pragma unroll
+      for (int k = j + 1; k < DM; ++k)
+        if (k < d) {
+          const double v = __shfl_sync(kFull, lij, k, GL);
+          if (k <= i) a[k] = fma(-lij, v, a[k]);
+        }
+    }
+  if (!fine) {
+#pragma unroll
+    for (int k = 0; k < DM; ++k) a[k] = (k == i) ? 1e-6 : 0.0;
+  }
+  return !fine || ok;
+}
+
 // Regularised Cholesky of the covariance in C (smem FP64, d x d):
 // chol(C + delta I), delta = 1e-10 tr(C)/d; if that fails, eigenvalues are
 // clipped at 1e-10 lambda_max first (section 2.1).  Work: smem FP64 [3 d d + d].
@@ -1683,97 +1747,137 @@ inline __device__ void reg_cholesky(int d, double* C, double* L, double* work, B
   __syncthreads();
 }
 
-// Mean and covariance (1/n) of the points j in [0, N) with member(j) true
-// (live_x [d][n_pad]), in one pass: coordinates are shifted by the first
-// member x_ref (so that E[(x - x_ref)(x - x_ref)^T] - (mu - x_ref)(mu -
-// x_ref)^T suffers no cancellation), products accumulate in FP32 within a
-// tile of kTile points and in FP64 across tiles.  tile: smem float
-// [d][kTileS] + d; acc: smem FP64 [d + d*d]; returns n.  Results: mean in
+// Row of packed lower-triangle entry e (e = a (a + 1) / 2 + b, b <= a < 32).
+__device__ __forceinline__ int packed_row(int e) {
+  int a = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+  if ((a + 1) * (a + 2) / 2 <= e) ++a;
+  if (a * (a + 1) / 2 > e) --a;
+  return a;
+}
+
+// Mean and covariance (1/N) of the points (live_x [d][n_pad]), in one pass:
+// coordinates are shifted by the first point x_ref (so that E[(x - x_ref)(x
+// - x_ref)^T] - (mu - x_ref)(mu - x_ref)^T suffers no cancellation), products
+// accumulate in FP32 within a tile of kTile points and in FP64 across tiles,
+// in their order.
+// A tile's sum of an entry is four packed chains over its points (points 2p,
+// 2p + 1 modulo 8).  A task is one chain of a 2 x 2 block of entries of one
+// tile (four loads feed four packed FMAs, two more on the diagonal add up
+// the rows for the mean), and moments_tiles(d) tiles are in shared memory
+// at once, so that a 256-thread block is busy at any d: one thread per
+// entry and one tile at a time had 65 of 256 threads busy at d = 10, and
+// half of the clustering phase's time was the barriers and loads between
+// tiles.
+// tile: smem float [tiles][d][kTileS], 16-byte aligned; part: smem float
+// [tiles][d + d (d + 1) / 2]; acc: smem FP64 [d + d*d].  Results: mean in
 // acc[0:d], covariance in acc[d:d+d*d].
-template <class Member>
-inline __device__ int node_moments(const float* __restrict__ live_x, int n_pad, int N, int d, Member member,
-                                   float* tile, double* acc, BlockScratch& S) {
+__host__ __device__ constexpr int moments_tiles(int d) {
+  const int dp = (d + 1) / 2, nb = dp * (dp + 1) / 2;
+  int t = 256 / (4 * nb);
+  const int room = 24 * 1024 / (d * kTileS * 4);
+  t = t < room ? t : room;
+  return t < 1 ? 1 : (t > 16 ? 16 : t);
+}
+__host__ __device__ constexpr int moments_part(int d, int tiles) { return tiles * (d + d * (d + 1) / 2); }
+
+inline __device__ void node_moments(const float* __restrict__ live_x, int n_pad, int N, int d, int tiles, float* tile,
+                                    float* part, double* acc) {
   const int tid = threadIdx.x, B = blockDim.x;
-  const int ne = d * (d + 1) / 2;
-  float* ref = tile + d * kTileS;
+  const int ne = d * (d + 1) / 2, dp = (d + 1) / 2, nb = dp * (dp + 1) / 2, row = d * kTileS;
   for (int i = tid; i < d + d * d; i += B) acc[i] = 0.0;
-  if (tid == 0) {
-    int j0 = 0;
-    while (j0 < N && !member(j0)) ++j0;
-    S.iw[0] = j0;
-  }
-  __syncthreads();
-  const int jr = S.iw[0];
-  for (int i = tid; i < d; i += B) ref[i] = (jr < N) ? live_x[(size_t)i * n_pad + jr] : 0.f;
-  __syncthreads();
-  int cnt = 0;
-  for (int j0 = 0; j0 < N; j0 += kTile) {
-    // eight loads in flight per thread before the first store (one at a
-    // time, the tile's loads were most of the clustering phase)
-    for (int q0 = tid; q0 < d * kTile; q0 += 8 * B) {
-      float v[8];
+  for (int j0 = 0; j0 < N; j0 += tiles * kTile) {
+    const int nt = min(tiles, (N - j0 + kTile - 1) / kTile);
+    // a warp per row (one coordinate of one tile): four points per lane, up
+    // to four rows in flight
+    constexpr int kFly = 4;
+    const int lane = tid & 31, nw = B >> 5, nrow = nt * d;
+    for (int r0 = tid >> 5; r0 < nrow; r0 += kFly * nw) {
+      float v[kFly][4], ref[kFly];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int q = q0 + u * B;
-        const int i = q / kTile, jj = q % kTile, j = j0 + jj;
-        v[u] = (q < d * kTile && j < N && member(j)) ? live_x[(size_t)i * n_pad + j] - ref[i] : 0.f;
+      for (int u = 0; u < kFly; ++u) {
+        const int r = min(r0 + u * nw, nrow - 1), t = r / d;
+        const float* src = live_x + (size_t)(r - t * d) * n_pad;
+        const int j = j0 + t * kTile + lane;
+        ref[u] = src[0];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[u][k] = j + 32 * k < N ? src[j + 32 * k] : ref[u];
       }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int q = q0 + u * B;
-        if (q < d * kTile) tile[(q / kTile) * kTileS + q % kTile] = v[u];
+      for (int u = 0; u < kFly; ++u)
+        if (r0 + u * nw < nrow) {
+          float* to = tile + (r0 + u * nw) * kTileS + lane;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) to[32 * k] = v[u][k] - ref[u];
+        }
+    }
+    __syncthreads();
+    const int tasks = 4 * nb * nt;
+    for (int q = tid; q < ((tasks + 31) & ~31); q += B) {
+      const int qq = min(q, tasks - 1), p = qq & 3, e = (qq >> 2) % nb, t = (qq >> 2) / nb;
+      const int A = packed_row(e), Bc = e - A * (A + 1) / 2;
+      const int a0 = 2 * A, a1 = min(a0 + 1, d - 1), b0 = 2 * Bc, b1 = min(b0 + 1, d - 1);
+      const float* base = tile + t * row + 2 * p;
+      const float* pa0 = base + a0 * kTileS;
+      const float* pa1 = base + a1 * kTileS;
+      const float* pb0 = base + b0 * kTileS;
+      const float* pb1 = base + b1 * kTileS;
+      float2 s00 = f2(0.f, 0.f), s01 = s00, s10 = s00, s11 = s00, m0 = s00, m1 = s00;
+#pragma unroll 8
+      for (int jj = 0; jj < kTile; jj += 8) {
+        const float2 x0 = ld2(pa0 + jj), x1 = ld2(pa1 + jj), y0 = ld2(pb0 + jj), y1 = ld2(pb1 + jj);
+        s00 = __ffma2_rn(x0, y0, s00);
+        s01 = __ffma2_rn(x0, y1, s01);
+        s10 = __ffma2_rn(x1, y0, s10);
+        s11 = __ffma2_rn(x1, y1, s11);
+        m0 = __fadd2_rn(x0, m0);
+        m1 = __fadd2_rn(x1, m1);
+      }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {  // (chain 0 + chain 1) + (chain 2 + chain 3)
+        auto add = [&](float2& s) {
+          s = __fadd2_rn(s, f2(__shfl_xor_sync(kFull, s.x, o), __shfl_xor_sync(kFull, s.y, o)));
+        };
+        add(s00);
+        add(s01);
+        add(s10);
+        add(s11);
+        add(m0);
+        add(m1);
+      }
+      if (p == 0 && q < tasks) {
+        float* out = part + t * (ne + d);
+        out[a0 * (a0 + 1) / 2 + b0] = s00.x + s00.y;
+        if (A != Bc) out[a0 * (a0 + 1) / 2 + b1] = s01.x + s01.y;
+        if (a1 > a0) {
+          out[a1 * (a1 + 1) / 2 + b0] = s10.x + s10.y;
+          out[a1 * (a1 + 1) / 2 + b1] = s11.x + s11.y;
+        }
+        if (A == Bc) {
+          out[ne + a0] = m0.x + m0.y;
+          if (a1 > a0) out[ne + a1] = m1.x + m1.y;
+        }
       }
     }
-    if (tid < kTile) cnt += (j0 + tid < N && member(j0 + tid)) ? 1 : 0;
     __syncthreads();
     for (int e = tid; e < ne + d; e += B) {
-      if (e < ne) {
-        int a = 0;
-        while ((a + 1) * (a + 2) / 2 <= e) ++a;
-        const int bcol = e - a * (a + 1) / 2;
-        const float* ta = tile + a * kTileS;
-        const float* tb = tile + bcol * kTileS;
-        // four independent packed accumulators
-        float2 s0 = f2(0.f, 0.f), s1 = s0, s2 = s0, s3 = s0;
-#pragma unroll 4
-        for (int jj = 0; jj < kTile; jj += 8) {
-          s0 = __ffma2_rn(ld2(ta + jj), ld2(tb + jj), s0);
-          s1 = __ffma2_rn(ld2(ta + jj + 2), ld2(tb + jj + 2), s1);
-          s2 = __ffma2_rn(ld2(ta + jj + 4), ld2(tb + jj + 4), s2);
-          s3 = __ffma2_rn(ld2(ta + jj + 6), ld2(tb + jj + 6), s3);
-        }
-        s0 = __fadd2_rn(__fadd2_rn(s0, s1), __fadd2_rn(s2, s3));
-        acc[d + a * d + bcol] += (double)(s0.x + s0.y);
-      } else {
-        const float* ta = tile + (e - ne) * kTileS;
-        float2 s0 = f2(0.f, 0.f), s1 = s0, s2 = s0, s3 = s0;
-#pragma unroll 4
-        for (int jj = 0; jj < kTile; jj += 8) {
-          s0 = __fadd2_rn(ld2(ta + jj), s0);
-          s1 = __fadd2_rn(ld2(ta + jj + 2), s1);
-          s2 = __fadd2_rn(ld2(ta + jj + 4), s2);
-          s3 = __fadd2_rn(ld2(ta + jj + 6), s3);
-        }
-        s0 = __fadd2_rn(__fadd2_rn(s0, s1), __fadd2_rn(s2, s3));
-        acc[e - ne] += (double)(s0.x + s0.y);
-      }
+      const int a = packed_row(min(e, ne - 1)), bcol = e - a * (a + 1) / 2;
+      double* to = acc + (e < ne ? d + a * d + bcol : e - ne);
+      double v = *to;
+      for (int t = 0; t < nt; ++t) v += (double)part[t * (ne + d) + e];
+      *to = v;
     }
     __syncthreads();
   }
-  const int n = (int)block_sum_ll(cnt, S);
-  const double inv = n > 0 ? 1.0 / n : 0.0;
+  const double inv = N > 0 ? 1.0 / N : 0.0;
   for (int e = tid; e < ne; e += B) {
-    int a = 0;
-    while ((a + 1) * (a + 2) / 2 <= e) ++a;
-    const int bcol = e - a * (a + 1) / 2;
+    const int a = packed_row(e), bcol = e - a * (a + 1) / 2;
     const double v = acc[d + a * d + bcol] * inv - (acc[a] * inv) * (acc[bcol] * inv);
     acc[d + a * d + bcol] = v;
     acc[d + bcol * d + a] = v;
   }
   __syncthreads();
-  for (int i = tid; i < d; i += B) acc[i] = acc[i] * inv + (double)ref[i];
+  for (int i = tid; i < d; i += B) acc[i] = acc[i] * inv + (double)live_x[(size_t)i * n_pad];
   __syncthreads();
-  return n;
 }
 
 }  // namespace nsd

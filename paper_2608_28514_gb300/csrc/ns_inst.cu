@@ -1,10 +1,15 @@
 // ns_inst.cu -- instantiates the per-dimension kernels for one register
 // class (compiled once per class with -DNS_DMAX=<class>, so the classes
-// build in parallel).
+// build in parallel; the wide classes in parts, -DNS_PART=<bits>: 1 the group
+// walkers' run kernel, 2 the thread walkers', 4 the rest).
 #include "ns_run.cuh"
 
 #ifndef NS_DMAX
 #error "compile with -DNS_DMAX=<register class>"
+#endif
+
+#ifndef NS_PART
+#define NS_PART 7
 #endif
 
 namespace nsd {
@@ -16,11 +21,11 @@ namespace nsd {
 // r*cluster + cluster - 1 are run r's).
 template <class K>
 static cudaError_t launch_runs(K* kernel, const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk,
-                               int vb, int cluster, cudaStream_t s) {
+                               int vb, int cluster, int room, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (cluster <= 1) {
-    kernel<<<n, block, smem, s>>>(runs, ids, chunk, vb);
+    kernel<<<n, block, smem, s>>>(runs, ids, chunk, vb, room);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
@@ -35,28 +40,47 @@ static cudaError_t launch_runs(K* kernel, const RunDesc* runs, const int* ids, i
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, runs, ids, chunk, vb);
+  return cudaLaunchKernelEx(&cfg, kernel, runs, ids, chunk, vb, room);
 }
 
-// The thread-walker kernel exists for the register classes whose walker (x,
-// v and a candidate in registers) fits 128 registers; the wider classes
-// always walk in groups.
-constexpr bool kHasThread = NS_DMAX <= kThreadWalkerMaxDim;
-
-cudaError_t NS_CAT(launch_run_, NS_DMAX)(const RunDesc* runs, const int* ids, int n, int block, size_t smem,
-                                         int chunk, int vb, int group, int cluster, cudaStream_t s) {
-  if constexpr (kHasThread)
-    if (!group) return launch_runs(k_run<NS_DMAX, kModeThread>, runs, ids, n, block, smem, chunk, vb, 1, s);
-  return launch_runs(k_run<NS_DMAX, kModeGroup>, runs, ids, n, block, smem, chunk, vb, cluster, s);
-}
-
-cudaError_t NS_CAT(occupancy_run_, NS_DMAX)(int block, size_t smem, int group, int* blocks_per_sm) {
-  auto* kernel = k_run<NS_DMAX, kModeGroup>;
-  if constexpr (kHasThread)
-    if (!group) kernel = k_run<NS_DMAX, kModeThread>;
+template <class K>
+static cudaError_t occupancy(K* kernel, int block, size_t smem, int* blocks_per_sm) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, block, smem);
+}
+
+// One run kernel's launch, or (n = 0) its occupancy, by mode.
+using RunFn = cudaError_t(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk, int vb,
+                          int cluster, int room, int* blocks_per_sm, cudaStream_t s);
+RunFn NS_CAT(run_group_, NS_DMAX), NS_CAT(run_thread_, NS_DMAX);
+
+#if NS_PART & 1
+cudaError_t NS_CAT(run_group_, NS_DMAX)(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk,
+                                        int vb, int cluster, int room, int* blocks_per_sm, cudaStream_t s) {
+  if (n == 0) return occupancy(k_run<NS_DMAX, kModeGroup>, block, smem, blocks_per_sm);
+  return launch_runs(k_run<NS_DMAX, kModeGroup>, runs, ids, n, block, smem, chunk, vb, cluster, room, s);
+}
+#endif
+
+#if NS_PART & 2
+cudaError_t NS_CAT(run_thread_, NS_DMAX)(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk,
+                                         int vb, int, int room, int* blocks_per_sm, cudaStream_t s) {
+  if (n == 0) return occupancy(k_run<NS_DMAX, kModeThread>, block, smem, blocks_per_sm);
+  return launch_runs(k_run<NS_DMAX, kModeThread>, runs, ids, n, block, smem, chunk, vb, 1, room, s);
+}
+#endif
+
+#if NS_PART & 4
+cudaError_t NS_CAT(launch_run_, NS_DMAX)(const RunDesc* runs, const int* ids, int n, int block, size_t smem,
+                                         int chunk, int vb, int group, int cluster, int room, cudaStream_t s) {
+  return (group ? NS_CAT(run_group_, NS_DMAX) : NS_CAT(run_thread_, NS_DMAX))(runs, ids, n, block, smem, chunk, vb,
+                                                                             cluster, room, nullptr, s);
+}
+
+cudaError_t NS_CAT(occupancy_run_, NS_DMAX)(int block, size_t smem, int group, int* blocks_per_sm) {
+  return (group ? NS_CAT(run_group_, NS_DMAX) : NS_CAT(run_thread_, NS_DMAX))(nullptr, nullptr, 0, block, smem, 0, 0, 1,
+                                                                             0, blocks_per_sm, nullptr);
 }
 
 cudaError_t NS_CAT(launch_loglike_, NS_DMAX)(const LikParams& P, int n, const float* x, float* out,
@@ -90,8 +114,9 @@ cudaError_t NS_CAT(launch_slice_, NS_DMAX)(const LikParams& P, const SliceCfg& S
 // r*cluster + cluster - 1), which share its tensor-core evaluations.
 cudaError_t launch_run_mlp(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk, int cluster,
                            cudaStream_t s) {
-  return launch_runs(k_run<32, kModeMlp>, runs, ids, n, block, smem, chunk, block, cluster, s);
+  return launch_runs(k_run<32, kModeMlp>, runs, ids, n, block, smem, chunk, block, cluster, 0, s);
 }
+#endif
 #endif
 
 }  // namespace nsd

@@ -108,11 +108,13 @@ __global__ void k_evidence(int N, int n, const float* __restrict__ l, double* st
   }
 }
 
-__global__ void k_cluster(RunDesc R, uint32_t t) {
+// DM: a register class >= d.
+template <int DM>
+__global__ void __launch_bounds__(256) k_cluster(const RunDesc R, uint32_t t) {
   extern __shared__ __align__(16) char sm[];
   __shared__ BlockScratch S;
-  const Carve cv = make_carve(R.d, 1, R.n_nodes, kMaxDim, false, R.spill != 0);
-  cluster_phase(R, t, sm, cv, S, blockDim.x);
+  const Carve cv = make_carve(R.d, 1, R.n_nodes, kMaxDim, false, R.spill != 0, 0, R.N, kRunSmemBudget);
+  cluster_phase<DM, true>(R, t, sm, cv, S, blockDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -143,7 +145,7 @@ void set_err(std::string* dst, const char* fmt, ...) {
 
 struct ClassFns {
   int dmax;
-  cudaError_t (*run)(const RunDesc*, const int*, int, int, size_t, int, int, int, int, cudaStream_t);
+  cudaError_t (*run)(const RunDesc*, const int*, int, int, size_t, int, int, int, int, int, cudaStream_t);
   cudaError_t (*ll)(const LikParams&, int, const float*, float*, cudaStream_t);
   cudaError_t (*sl)(const LikParams&, const SliceCfg&, int, int, int, const float*, const float*, const int*,
                     const float*, const float*, const int*, float*, float*, float*, float*, int*, long long*, int*,
@@ -181,14 +183,11 @@ bool same_network(const ns_likelihood& a, const ns_likelihood& b) {
          eq(a.sigma_out, b.sigma_out, no);
 }
 
-// Dynamic shared memory a run kernel may take (the static part stays below 3 KB).
-constexpr size_t kRunSmemBudget = 227 * 1024 - 3072;
-
 // A run whose cluster tables do not fit in shared memory keeps them in
 // global memory (make_carve's spill).
 bool run_spills(const ns_problem& p, int n_nodes) {
   const bool mlp = p.lik->kind == NS_LIK_MLP;
-  return make_carve(p.d, p.m, n_nodes, dmax_class(p.d), mlp, false).total > kRunSmemBudget;
+  return make_carve(p.d, p.m, n_nodes, dmax_class(p.d), mlp, false).base > kRunSmemBudget;
 }
 
 // Global tree scratch of a spilled run, sized for the widest block (the MLP
@@ -239,71 +238,80 @@ int block_for_m(int m) {
 //
 // A walk is a chain of dependent likelihoods, so lanes beyond one per walker
 // shorten it (slice_walker_lanes) as long as the SMs are not already full of
-// walkers.  Every class starts with the block that one walker per thread
-// needs; while the runs' threads stay within what the SMs hold at 128
-// registers (512 each), the class whose runs take longest gets twice the
-// lanes, first a wider block, then a cluster of blocks on as many SMs, up to
-// eight lanes per walker on blocks of 128 busy threads.  A batch that fills
-// the GPU by itself keeps one walker per thread, unless its blocks leave at
-// least four lanes per walker idle anyway.
+// walkers.  Every class starts with one walker per thread, or with groups
+// where its smallest block leaves four lanes per walker idle anyway.  While
+// the runs' threads stay within what the SMs hold at 128 registers (512
+// each; a thread walker above 12 dimensions takes twice that), the class
+// whose runs take longest goes on to four lanes per walker, to eight, and
+// to blocks of no more than 128 busy lanes, on wider blocks first and then on
+// clusters of blocks.  (Two lanes per walker were no faster than one thread:
+// sixteen groups of a warp in lock step take the longest of their shrink
+// sequences.  266 runs of a 28-D mixture, m = 69: 33.3 ms against 30.5.)
 struct ClassNeed {
   int dmax, n, max_m, n_steps;  // runs, largest batch and slice steps of a class
 };
 struct RunShape {
-  int block, vb, group, cluster, group_w;
-  double est;  // relative time of an iteration's walk
+  int block, vb, group, cluster, group_w, room;
+  long long threads;  // of one run, at 128 registers
+  double est;         // relative time of an iteration's walk
 };
-void shape_lanes(const ClassNeed& c, RunShape& q) {
-  q.group_w = (c.max_m + q.cluster - 1) / q.cluster;
-  const int G = group_lanes(q.block, q.group_w);
-  // rounds of likelihoods per slice step, and their cost
-  const double rounds = G >= 8 ? 2.3 : (G >= 4 ? 3.0 : (G >= 2 ? 4.5 : 7.0));
+RunShape shape_at(const ClassNeed& c, int stage) {
+  RunShape q;
+  q.vb = q.block = block_for_m(c.max_m);
+  q.group = q.group_w = 0;
+  q.cluster = 1;
+  q.room = 0;
+  q.threads = q.block * (c.dmax > 12 ? 2 : 1);
+  double rounds = 7.0;  // of likelihoods per slice step
+  if (stage > 0) {
+    const int G = stage == 1 ? 4 : 8;
+    q.block = std::max(q.vb, std::min(256, (G * c.max_m + 31) / 32 * 32));
+    while (q.cluster < kGroupClusterMax && group_lanes(q.block, (c.max_m + q.cluster - 1) / q.cluster) < G)
+      q.cluster *= 2;
+    while (stage == 3 && q.cluster < kGroupClusterMax && 128 * q.cluster < 8 * c.max_m) q.cluster *= 2;
+    q.group = 1;
+    q.group_w = (c.max_m + q.cluster - 1) / q.cluster;
+    q.threads = q.block * q.cluster;
+    rounds = stage == 1 ? 3.0 : (stage == 2 ? 2.3 : 2.0);
+  }
   q.est = c.n_steps * rounds * (100.0 + 8.0 * c.dmax);
+  return q;
 }
 std::vector<RunShape> plan_shapes(const std::vector<ClassNeed>& need, int n_sm) {
-  std::vector<RunShape> out(need.size());
+  std::vector<RunShape> out;
+  std::vector<int> stage(need.size(), 0);
   long long threads = 0;
   for (size_t k = 0; k < need.size(); ++k) {
-    RunShape& q = out[k];
-    q.vb = q.block = block_for_m(need[k].max_m);
-    q.cluster = 1;
-    if (need[k].dmax > kThreadWalkerMaxDim) {  // no thread walkers: two lanes each at least
-      if (2 * need[k].max_m > q.block) q.block = 256;
-      if (2 * need[k].max_m > q.block) q.cluster = 2;
+    for (int s = 1; s <= 2; ++s) {
+      const RunShape q = shape_at(need[k], s);
+      if (q.cluster == 1 && q.block == q.vb) stage[k] = s;
     }
-    shape_lanes(need[k], q);
-    threads += (long long)need[k].n * q.block * q.cluster;
+    out.push_back(shape_at(need[k], stage[k]));
+    threads += need[k].n * out[k].threads;
   }
   const long long budget = 512LL * n_sm;
-  const bool roomy = threads <= budget / 2;
   std::vector<char> settled(need.size(), 0);
   for (;;) {
     int best = -1;
     for (size_t k = 0; k < need.size(); ++k)
       if (!settled[k] && (best < 0 || out[k].est > out[best].est)) best = (int)k;
     if (best < 0) break;
-    const ClassNeed& c = need[best];
-    RunShape q = out[best];
-    if (q.block < 256 && 8 * q.group_w > q.block) q.block = 256;
-    else if (q.cluster < kGroupClusterMax && 128 * q.cluster < 8 * c.max_m) q.cluster *= 2;
-    else settled[best] = 1;
-    const long long more = (long long)c.n * (q.block * q.cluster - out[best].block * out[best].cluster);
-    if (threads + more > budget) settled[best] = 1;
-    if (settled[best]) continue;
-    threads += more;
-    shape_lanes(c, q);
-    out[best] = q;
-  }
-  for (size_t k = 0; k < need.size(); ++k) {
-    RunShape& q = out[k];
-    const int G = group_lanes(q.block, q.group_w);
-    q.group = need[k].dmax > kThreadWalkerMaxDim || G >= (roomy ? 2 : 4);
-    if (!q.group) {
-      q.block = q.vb;
-      q.cluster = 1;
-      q.group_w = 0;
+    const RunShape q = shape_at(need[best], stage[best] + 1);
+    const long long more = need[best].n * (q.threads - out[best].threads);
+    if (stage[best] == 3 || threads + more > budget) {
+      settled[best] = 1;
+      continue;
     }
+    threads += more;
+    out[best] = q;
+    ++stage[best];
   }
+  // shared memory for staged points: the whole SM's where every block has one
+  // to itself, else its threads' share
+  long long blocks = 0;
+  for (size_t k = 0; k < need.size(); ++k) blocks += (long long)need[k].n * out[k].cluster;
+  for (RunShape& q : out)
+    q.room = !q.group ? 0 : (int)(blocks <= n_sm ? kRunSmemBudget : kRunSmemBudget * q.block / 512);
   return out;
 }
 
@@ -540,6 +548,7 @@ struct ClassGroup {
   int cluster = 1;  // CTAs per run
   int vb = 0;       // analytic runs: threads whose order the sums follow (RunShape)
   int group = 0;    // analytic runs: walkers are lane groups
+  int room = 0;     // shared memory a block may take to stage its points (make_carve)
   double est = 1e30;  // relative time of an iteration (MLP runs: the longest)
   bool mlp = false;
   size_t smem = 0;
@@ -548,7 +557,7 @@ struct ClassGroup {
 
 cudaError_t launch_class(const ClassGroup& g, const RunDesc* d_runs, int chunk, cudaStream_t s) {
   if (g.mlp) return launch_run_mlp(d_runs, g.d_ids, g.n, g.block, g.smem, chunk, g.cluster, s);
-  return kClasses[class_index(g.dmax)].run(d_runs, g.d_ids, g.n, g.block, g.smem, chunk, g.vb, g.group, g.cluster, s);
+  return kClasses[class_index(g.dmax)].run(d_runs, g.d_ids, g.n, g.block, g.smem, chunk, g.vb, g.group, g.cluster, g.room, s);
 }
 
 }  // namespace
@@ -909,10 +918,12 @@ ns_status ns_create_batch(int n_runs, const ns_problem* runs, const ns_options* 
       g.vb = q.vb;
       g.group = q.group;
       g.cluster = q.cluster;
+      g.room = q.room;
     }
     for (int r : members[ci])
       smem = std::max(smem, make_carve(runs[r].d, runs[r].m, n_nodes, g.dmax, g.mlp, off[r].spill != 0,
-                                       g.group ? (runs[r].m + g.cluster - 1) / g.cluster : 0)
+                                       g.group ? (runs[r].m + g.cluster - 1) / g.cluster : 0, runs[r].n_live,
+                                       (size_t)g.room)
                                 .total);
     if (g.mlp) {
       g.block = std::max(g.block, kMlpThreads);  // the BF16 evaluator's warp roles
@@ -1689,14 +1700,14 @@ ns_status ns_run_noalloc(const ns_problem* problem, const ns_options* opt_in, fl
   const RunDesc* d_desc = reinterpret_cast<const RunDesc*>(base + o_desc);
   const int* d_ids = reinterpret_cast<const int*>(base + o_ids);
   const RunShape q = plan_shapes({{dmax_class(d), 1, m, p.n_slice_steps}}, device_sms())[0];
-  const size_t smem = make_carve(d, m, n_nodes, dmax_class(d), false, spill, q.group_w).total;
+  const size_t smem = make_carve(d, m, n_nodes, dmax_class(d), false, spill, q.group_w, N, (size_t)q.room).total;
   const int chunk = opt.chunk_iters > 0 ? opt.chunk_iters : 1000;
   const long long max_rounds = opt.max_iter / chunk + 2;
   RunState hs;
   std::memset(&hs, 0, sizeof(hs));
   for (long long round = 0;; ++round) {
     const cudaError_t e =
-        kClasses[class_index(d)].run(d_desc, d_ids, 1, q.block, smem, chunk, q.vb, q.group, q.cluster, s);
+        kClasses[class_index(d)].run(d_desc, d_ids, 1, q.block, smem, chunk, q.vb, q.group, q.cluster, q.room, s);
     NS_CUDA(e, nullptr);
     NS_CUDA(cudaMemcpyAsync(&hs, base + o_state, sizeof(RunState), cudaMemcpyDeviceToHost, s), nullptr);
     NS_CUDA(cudaStreamSynchronize(s), nullptr);
@@ -1924,17 +1935,18 @@ ns_status ns_cluster(int N, int n_pad, int d, const float* live_x, const ns_opti
     R.wsp = static_cast<float*>(scratch);
     R.side = reinterpret_cast<int*>(static_cast<char*>(scratch) + sizeof(float) * (size_t)d * n_pad);
   }
-  if (opt.depth > 0 && make_carve(d, 1, R.n_nodes, kMaxDim).total > 227 * 1024) {
+  if (opt.depth > 0 && make_carve(d, 1, R.n_nodes, kMaxDim).base > 227 * 1024) {
     R.spill = 1;
     R.tree_ws = static_cast<char*>(scratch) + cluster_points_bytes(N, n_pad, d);
   }
-  const size_t smem = make_carve(d, 1, R.n_nodes, kMaxDim, false, R.spill != 0).total;
+  const size_t smem = make_carve(d, 1, R.n_nodes, kMaxDim, false, R.spill != 0, 0, N, kRunSmemBudget).total;
   if (smem > 227 * 1024) {
     set_err(nullptr, "ns_cluster: %zu bytes of shared memory needed (limit 227 KB)", smem);
     return NS_ERR_ARG;
   }
-  NS_CUDA(cudaFuncSetAttribute(k_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), nullptr);
-  k_cluster<<<1, 256, smem, (cudaStream_t)stream>>>(R, t);
+  auto* kernel = d <= 4 ? k_cluster<4> : (d <= 8 ? k_cluster<8> : (d <= 16 ? k_cluster<16> : k_cluster<32>));
+  NS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), nullptr);
+  kernel<<<1, 256, smem, (cudaStream_t)stream>>>(R, t);
   NS_CUDA(cudaGetLastError(), nullptr);
   return NS_OK;
 }

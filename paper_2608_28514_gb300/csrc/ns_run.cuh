@@ -85,7 +85,12 @@ struct RunDesc {
 // device from the run's sizes.
 struct Carve {
   size_t lik, scr, sel, chol, cent, mask, worst, W, seed, sel_slot, sel_key, candA, candB, candT, list, vals, slots,
-      ctr, stage_cid, xbuf, lbuf, rlist, tile, acc, c64, l64, work, tree, mlp, total;
+      ctr, stage_cid, xbuf, lbuf, rlist, tile, acc, c64, l64, work, tree, hot, pbuf, stage, mom, mlp, total;
+  size_t base;       // the total without the slot sums' buffer (what decides whether a run spills)
+  int rows;          // rows (slots x items) of that buffer, per warp
+  int tiles;         // tiles of the moments in shared memory at once
+  size_t work_bytes; // bytes at pbuf that the eigen-clips may use
+  bool staged;       // the tree works on points staged in shared memory
   bool chol_global;  // the cluster Cholesky factors live in global memory (MLP runs, spilled runs)
   bool tree_global;  // the cluster-tree scratch lives in global memory (spilled runs)
 };
@@ -94,6 +99,9 @@ struct Carve {
 // three weight-tile stages.
 constexpr int kRunMlpStages = 3;
 using RunMlpSmem = MlpSmem<kMlpNbMax, kRunMlpStages>;
+
+// Dynamic shared memory a run kernel may take (the static part stays below 3 KB).
+constexpr size_t kRunSmemBudget = 227 * 1024 - 3072;
 
 __host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
 
@@ -104,9 +112,11 @@ __host__ __device__ constexpr int mlp_xs(int d) { return (d + 3) & ~3; }
 // deep tree); the Cholesky factors and the tree scratch then stay in global
 // memory (only the clustering and the direction draws read them).
 // group_w: walkers of one block when a walker is a group of lanes
-// (slice_walker_lanes), 0 when it is a thread.
+// (slice_walker_lanes), 0 when it is a thread.  room: shared memory the block
+// may take to stage its N live points for the cluster tree (with the factors
+// of a spilled run), 0 for none.
 __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax, bool mlp = false,
-                                            bool spill = false, int group_w = 0) {
+                                            bool spill = false, int group_w = 0, int N = 0, size_t room = 0) {
   Carve c;
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -149,35 +159,83 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
   c.work = take(sizeof(double) * (3 * d * d + d));
   // per-warp partials for every warp of the block (MLP blocks have kMlpThreads threads, others <= 256)
   c.tree = take(c.tree_global ? 0 : tree_bytes(d, n_nodes, mlp ? kMlpThreads / 32 : 8, tree_chol_warps(d, 8)));
+  const int nwt = mlp ? kMlpThreads / 32 : 8, nwc = tree_chol_warps(d, 8);
+  const size_t end_tree = o;
   c.mlp = phase0;
+  size_t other = phase0;  // the end of what the clustering scratch shares its space with
+  o = phase0;
   if (!mlp) {
-    const size_t end_cluster = o;
-    o = phase0;
     c.slots = take(group_w > 0 ? sizeof(float) * (size_t)group_floats(dmax) * group_w
                                : sizeof(float) * (size_t)dir_row(dmax) * (m + 31) / 32 * 32);
-    const size_t end_slots = o;
-    o = phase0;
-    c.candA = take(cand_bytes);
-    c.candB = take(cand_bytes);
-    c.candT = take(cand_bytes);
-    if (end_cluster > o) o = end_cluster;
-    if (end_slots > o) o = end_slots;
+    other = o;
   } else {
     c.slots = phase0;
-    const size_t end_cluster = o;
-    o = phase0;
-    c.candA = take(cand_bytes);
-    c.candB = take(cand_bytes);
-    c.candT = take(cand_bytes);
-    const size_t end_cand = o;
     const size_t end_bf16 = phase0 + RunMlpSmem::kBytes + 1024;  // + alignment of the tensor-core region
     const size_t end_f32 = phase0 + mlp_f32_act_bytes(kMlpF32NbWide);
-    o = end_cluster;
-    if (end_cand > o) o = end_cand;
-    if (end_bf16 > o) o = end_bf16;
-    if (end_f32 > o) o = end_f32;
+    other = end_bf16 > end_f32 ? end_bf16 : end_f32;
   }
-  c.total = o;
+  o = phase0;
+  c.candA = take(cand_bytes);
+  c.candB = take(cand_bytes);
+  c.candT = take(cand_bytes);
+  if (o > other) other = o;
+  c.base = end_tree > other ? end_tree : other;
+  // the splits' tables of a spilled run; the slot sums' buffer (slot_sums) and
+  // the staged points; the moments' tiles, over the scratch used after them
+  o = end_tree;
+  c.hot = spill ? take(tree_hot_bytes(d, n_nodes, nwt)) : c.tree;
+  const size_t at = o;
+  auto sums = [&](int rows) { return al16(sizeof(float) * (size_t)nwt * rows * 33); };
+  size_t grown = at;
+  c.rows = kSumRows;
+  c.pbuf = c.stage = at;
+  c.work_bytes = 0;
+  c.staged = false;
+  if (n_nodes > 1) {
+    const size_t pts = al16(sizeof(float) * (size_t)d * N), st = pts + al16(N);
+    const size_t own_chol = spill && !mlp ? al16(sizeof(float) * (size_t)n_nodes * d * d) : 0;
+    for (int rows = kSumRows; rows >= 16 && !c.staged; rows /= 2) {
+      size_t end = at + sums(rows) + st;
+      if (end < other) end = other;
+      if (!mlp && end + own_chol <= room) {
+        c.staged = true;
+        c.rows = rows;
+        c.stage = at + sums(rows);
+        c.work_bytes = sums(rows) + pts;
+        grown = at + sums(rows) + st;
+        if (spill) {
+          c.chol = end;
+          c.chol_global = false;
+          grown = end + own_chol;
+        }
+      }
+    }
+    if (!c.staged) {
+      const size_t work = sizeof(double) * (size_t)nwc * (5 * d * d + d);
+      if (!spill && at + sums(c.rows) > kRunSmemBudget) {  // in the factorisation's work space
+        while (c.rows > 1 && sums(c.rows) > work) c.rows /= 2;
+        c.pbuf = end_tree - al16(work);
+        c.work_bytes = al16(work);
+      } else {
+        c.work_bytes = sums(c.rows) > al16(work) ? sums(c.rows) : al16(work);
+        grown = at + c.work_bytes;
+        if (grown > kRunSmemBudget) {
+          c.work_bytes = sums(c.rows);
+          grown = at + c.work_bytes;
+        }
+      }
+    }
+  }
+  c.tiles = moments_tiles(d);
+  o = c.c64;
+  c.mom = take(sizeof(float) * ((size_t)c.tiles * d * kTileS + moments_part(d, c.tiles)));
+  if (o > kRunSmemBudget || (spill && c.staged && o > c.chol)) {  // one tile in its own place, its sums where the factorisation will work
+    c.tiles = 1;
+    c.mom = c.tile;
+  } else if (o > grown) {
+    grown = o;
+  }
+  c.total = grown > other ? grown : other;
   return c;
 }
 
@@ -212,9 +270,10 @@ inline __device__ void init_live(const RunDesc& R, const LikParams& P) {
 // a3 (section 2.1): the root node is the whole live set (mean, covariance,
 // regularised FP64 Cholesky); for depth >= 1 the tree of cluster_tree
 // follows.
-inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, const Carve& cv, BlockScratch& S, int vb) {
+// STAGE: the kernel has the variant that stages the points.
+template <int DM, bool STAGE>
+__device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, const Carve& cv, BlockScratch& S, int vb) {
   const int d = R.d;
-  float* tile = reinterpret_cast<float*>(sm + cv.tile);
   double* acc = reinterpret_cast<double*>(sm + cv.acc);
   double* C64 = reinterpret_cast<double*>(sm + cv.c64);
   double* L64 = reinterpret_cast<double*>(sm + cv.l64);
@@ -222,10 +281,29 @@ inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, con
   float* s_chol = cv.chol_global ? R.chol : reinterpret_cast<float*>(sm + cv.chol);
   float* s_cent = reinterpret_cast<float*>(sm + cv.cent);
   int* s_mask = reinterpret_cast<int*>(sm + cv.mask);
-  const int n = node_moments(R.live_x, R.n_pad, R.N, d, [](int) { return true; }, tile, acc, S);
-  for (int i = threadIdx.x; i < d * d; i += blockDim.x) C64[i] = acc[d + i];
+  const int n = R.N;
+  float* mom = reinterpret_cast<float*>(sm + cv.mom);
+  node_moments(R.live_x, R.n_pad, R.N, d, cv.tiles, mom,
+               cv.mom == cv.tile ? reinterpret_cast<float*>(work) : mom + (size_t)cv.tiles * d * kTileS, acc);
+  if (threadIdx.x < 32) {
+    const int i = threadIdx.x;
+    double a[DM];
+#pragma unroll
+    for (int k = 0; k < DM; ++k) a[k] = (i < d && k <= i) ? acc[d + i * d + k] : 0.0;
+    const int ok = reg_chol_rows<DM>(d, i % chol_lanes(DM), a);
+#pragma unroll
+    for (int k = 0; k < DM; ++k)
+      if (i < d && k < d) L64[i * d + k] = k <= i ? a[k] : 0.0;
+    if (i == 0) S.iw[0] = ok;
+  }
   __syncthreads();
-  reg_cholesky(d, C64, L64, work, S);
+  const int chol_ok = S.iw[0];
+  __syncthreads();
+  if (!chol_ok) {  // the eigen-clip
+    for (int i = threadIdx.x; i < d * d; i += blockDim.x) C64[i] = acc[d + i];
+    __syncthreads();
+    reg_cholesky(d, C64, L64, work, S);
+  }
   for (int i = threadIdx.x; i < d * d; i += blockDim.x) {
     const float f = (float)L64[i];
     s_chol[i] = f;
@@ -244,7 +322,7 @@ inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, con
     unsigned* m2u = reinterpret_cast<unsigned*>(&S.iw[0]);
     if (threadIdx.x == 0) *m2u = 0u;
     __syncthreads();
-    const unsigned mx = max_mahalanobis2(R.live_x, R.n_pad, R.N, d, s_chol, s_cent);
+    const unsigned mx = max_mahalanobis2<DM>(R.live_x, R.n_pad, R.N, d, s_chol, s_cent);
     atomicMax(m2u, mx);
     __syncthreads();
     const float rad = sqrtf(__uint_as_float(*m2u));
@@ -268,14 +346,14 @@ inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, con
     return;
   }
   const int nw = blockDim.x >> 5;
-  const int nw_chol = tree_chol_warps(d, 8) < nw ? tree_chol_warps(d, 8) : nw;
-  const TreeScratch T = tree_carve(cv.tree_global ? R.tree_ws : sm + cv.tree, d, R.n_nodes, nw, tree_chol_warps(d, 8));
+  const TreeScratch T =
+      tree_carve(cv.tree_global ? R.tree_ws : sm + cv.tree, sm + cv.hot, d, R.n_nodes, nw, tree_chol_warps(d, 8));
   if (threadIdx.x == 0) T.node_n[0] = n;
   __syncthreads();
   TreeIO io;
   io.x = R.live_x;
   io.y = R.wsp;
-  io.side = R.side;
+  io.side = reinterpret_cast<uint8_t*>(R.side);
   io.N = R.N;
   io.n_pad = R.n_pad;
   io.d = d;
@@ -299,7 +377,17 @@ inline __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, con
   io.s_mask = s_mask;
   io.bracket = R.bracket;
   io.vb = vb;
-  cluster_tree(io, T, S, nw_chol);
+  io.pbuf = reinterpret_cast<float*>(sm + cv.pbuf);
+  io.rows = cv.rows;
+  io.stage = reinterpret_cast<float*>(sm + cv.stage);
+  io.work_bytes = cv.work_bytes;
+  if constexpr (STAGE) {
+    if (cv.staged) {
+      cluster_tree<DM, true>(io, T, S);
+      return;
+    }
+  }
+  cluster_tree<DM, false>(io, T, S);
 }
 
 inline __device__ int nearest_leaf(const float* x, int d, int n_nodes, const float* cent, const int* mask) {
@@ -325,8 +413,8 @@ inline __device__ int nearest_leaf(const float* x, int d, int n_nodes, const flo
 // so that its registers are allocated apart from the rest of the run kernel.
 template <int DMAX>
 __device__ __noinline__ void walker_phase(const RunDesc& R, const LikParams& P, const SliceCfg& SC,
-                                          const float* s_W, const int* s_seed, const float* s_chol, float* s_slots,
-                                          long long& ev, int& fl, long long& cyc_draw, long long& cyc_walk) {
+                                          const float* s_W, const int* s_seed, float* s_slots, long long& ev, int& fl,
+                                          long long& cyc_walk) {
   const int tid = threadIdx.x, m = R.m, d = R.d;
   const bool act = tid < m;
   const int i = act ? tid : 0;
@@ -347,7 +435,6 @@ __device__ __noinline__ void walker_phase(const RunDesc& R, const LikParams& P, 
                      thr_out, thr_in, O, e, f);
   ev = act ? e : 0;
   fl = act ? f : 0;
-  cyc_draw = 0;  // the draws happen before, block-wide (k_run)
   cyc_walk = clock64() - c1;
 }
 
@@ -1111,30 +1198,31 @@ inline __device__ void init_live_mlp(const RunDesc& R, float* xbuf, float* lbuf,
   }
 }
 
-// How a run's walkers sit on its block: one per thread (the small register
-// classes, when the runs fill the GPU), the lock-step rounds of an MLP run,
-// or a group of lanes each (and, with few runs, a cluster of blocks per run).
+// How a run's walkers sit on its block: one per thread (when the runs fill
+// the GPU), the lock-step rounds of an MLP run, or a group of lanes each (and,
+// with few runs, a cluster of blocks per run).
 enum RunMode { kModeThread = 0, kModeMlp = 1, kModeGroup = 2 };
-constexpr int kThreadWalkerMaxDim = 12;  // widest register class with a thread-walker kernel
 
-// Blocks of up to 256 threads, 128 registers per thread (two such blocks,
-// or four of 128 threads, per SM).  NS_RUN_MINB and NS_RUN_MAXNREG (build
-// time) override the cap of the thread-walker kernels.
+// Blocks of up to 256 threads.  128 registers per thread (two such blocks, or
+// four of 128 threads, per SM), but for the thread walkers of the wide
+// register classes, which keep a point, a direction and a candidate in
+// registers.  NS_RUN_MINB and NS_RUN_MAXNREG (build time) override the cap of
+// the thread-walker kernels.
 #ifdef NS_RUN_MINB
-#define NS_MINB(MODE) ((MODE) == kModeThread ? NS_RUN_MINB : 2)
+#define NS_MINB(MODE, D) ((MODE) == kModeThread ? NS_RUN_MINB : 2)
 #else
-#define NS_MINB(MODE) 2
+#define NS_MINB(MODE, D) ((MODE) == kModeThread && (D) > 12 ? 1 : 2)
 #endif
 #ifdef NS_RUN_MAXNREG
-#define NS_RUN_BOUNDS(MODE)                                \
+#define NS_RUN_BOUNDS(MODE, D)                             \
   __launch_bounds__(((MODE) == kModeMlp ? kMlpThreads : 256)) \
       __maxnreg__((MODE) == kModeMlp ? 200 : ((MODE) == kModeThread ? NS_RUN_MAXNREG : 128))
 #else
-#define NS_RUN_BOUNDS(MODE) \
-  __launch_bounds__(((MODE) == kModeMlp ? kMlpThreads : 256), ((MODE) == kModeMlp ? 1 : NS_MINB(MODE)))
+#define NS_RUN_BOUNDS(MODE, D) \
+  __launch_bounds__(((MODE) == kModeMlp ? kMlpThreads : 256), ((MODE) == kModeMlp ? 1 : NS_MINB(MODE, D)))
 #endif
 template <int DMAX, int MODE>
-__global__ void NS_RUN_BOUNDS(MODE) k_run(const RunDesc* __restrict__ runs, const int* __restrict__ ids, int chunk, int vb) {
+__global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs, const int* __restrict__ ids, int chunk, int vb, int room) {
   constexpr bool MLP = MODE == kModeMlp;
   extern __shared__ __align__(16) char sm[];
   __shared__ RunDesc R;
@@ -1171,7 +1259,7 @@ __global__ void NS_RUN_BOUNDS(MODE) k_run(const RunDesc* __restrict__ runs, cons
   __syncthreads();
   const int d = R.d, N = R.N, m = R.m;
   const Carve cv = make_carve(d, m, R.n_nodes, DMAX, MLP, R.spill != 0,
-                              MODE == kModeGroup ? (m + (int)C - 1) / (int)C : 0);
+                              MODE == kModeGroup ? (m + (int)C - 1) / (int)C : 0, N, (size_t)room);
   if constexpr (MLP) {
     if (rank > 0) {
       mlp_follower(R, &mlp_ctx, mail, align1024_shared(sm + cv.mlp), C, rank);
@@ -1275,7 +1363,7 @@ __global__ void NS_RUN_BOUNDS(MODE) k_run(const RunDesc* __restrict__ runs, cons
     };
     // a3: clustering
     const bool reclustered = R.recluster_every > 0 && (t % (uint32_t)R.recluster_every) == 0;
-    if (reclustered) cluster_phase(R, t, sm, cv, S, vb);
+    if (reclustered) cluster_phase<DMAX, MODE == kModeGroup>(R, t, sm, cv, S, vb);
     tick(kPhCluster);
     // a1-a2: selection
     select_worst(R.live_l, N, m, R.k0, R.k1, t, s_sel_slot, s_sel_key, s_worst, s_W, s_seed, X, S);
@@ -1321,7 +1409,7 @@ __global__ void NS_RUN_BOUNDS(MODE) k_run(const RunDesc* __restrict__ runs, cons
         walker_phase_warp<DMAX>(R, P, SC, s_W, s_seed, 0, m, ev, fl);
         cyc_reeval = clock64() - cd1;
       } else if ((tid & ~31) < m) {
-        walker_phase<DMAX>(R, P, SC, s_W, s_seed, s_chol, s_slots, ev, fl, cyc_eval, cyc_reeval);
+        walker_phase<DMAX>(R, P, SC, s_W, s_seed, s_slots, ev, fl, cyc_reeval);
         if (R.wk_evals && tid < m) {
           R.wk_evals[tid] = (int)ev;
           R.wk_flags[tid] = fl;
@@ -1555,7 +1643,7 @@ __global__ void k_slice_warp(const LikParams P, SliceCfg SC, int m, int n_pad, i
 // Launchers, one set per class (defined in ns_inst.cu).
 #define NS_DECLARE_LAUNCHERS(D)                                                                          \
   cudaError_t launch_run_##D(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk, \
-                             int vb, int group, int cluster, cudaStream_t s);                                                            \
+                             int vb, int group, int cluster, int room, cudaStream_t s);                                                            \
   cudaError_t launch_loglike_##D(const LikParams& P, int n, const float* x, float* out, cudaStream_t s);  \
   cudaError_t launch_slice_##D(const LikParams& P, const SliceCfg& SC, int m, int n_pad, int correction,   \
                                const float* live_x, const float* live_l, const int* seed_slot,           \

@@ -1,7 +1,7 @@
 """The lane-group walkers (several lanes and several SMs per run) against the
 other shapes of the same run: a run alone takes up to eight lanes per walker on
-a cluster of blocks, the same run in a batch that fills the GPU one thread
-(up to 12 dimensions) or two lanes per walker.  Every shape takes the same
+a cluster of blocks, the same run in a batch that fills the GPU one thread per
+walker, and one in between something in between.  Every shape takes the same
 FP32 operations in the same order, so all of a run's buffers are equal bit
 for bit: the tolerance is zero."""
 import numpy as np

@@ -316,42 +316,6 @@ __device__ __forceinline__ int block_exclusive_scan(int v, BlockScratch& S, int*
   return base + x - v;
 }
 
-__device__ __forceinline__ double block_sum_d(double v, BlockScratch& S) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
-  if (lane == 0) S.dw[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    double w = lane < nw ? S.dw[lane] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_down_sync(kFull, w, o);
-    if (lane == 0) S.dw[32] = w;
-  }
-  __syncthreads();
-  const double r = S.dw[32];
-  __syncthreads();
-  return r;
-}
-
-__device__ __forceinline__ double block_max_d(double v, BlockScratch& S) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(kFull, v, o));
-  if (lane == 0) S.dw[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    double w = lane < nw ? S.dw[lane] : -CUDART_INF;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w = fmax(w, __shfl_down_sync(kFull, w, o));
-    if (lane == 0) S.dw[32] = w;
-  }
-  __syncthreads();
-  const double r = S.dw[32];
-  __syncthreads();
-  return r;
-}
-
 __device__ __forceinline__ float block_max_f(float v, BlockScratch& S) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
@@ -402,21 +366,101 @@ struct SelectScratch {
   int found[4];
 };
 
-// sel_slot/sel_key: smem [m] scratch.  Outputs (any address space): worst[m]
-// ascending by (logL, slot), W[m], seed_slot[m].
+// The start slot of walker i: the idx-th survivor in ascending slot order;
+// sel (the m selected slots, ascending) is skipped: sel[q] - q never falls, so
+// the number of selected slots at or below the answer is found by halving.
+__device__ __forceinline__ int survivor_slot(uint32_t k0, uint32_t k1, uint32_t t, int i, int N, int m, const int* sel) {
+  const int s = u_index(draw_at(k0, k1, t, (uint32_t)i, kPurposeSeed, 0), N - m);
+  int lo = 0, hi = m;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (sel[mid] - mid <= s) lo = mid + 1;
+    else hi = mid;
+  }
+  return s + lo;
+}
+
+// sel_slot/sel_key: smem [m] scratch.  keys: smem [N], or null (the log L are
+// then read from global memory in every pass).  Outputs (any address space):
+// worst[m] ascending by (logL, slot), W[m], seed_slot[m].
+//
+// The keys of a live set share their sign and most of their exponent, so
+// the radix select starts at the highest bit in which the smallest and the
+// largest key differ, and stops as soon as a digit's bucket is taken whole;
+// one pass or two of eight bits instead of four.  One worst point (m = 1) is a
+// minimum.  (N = 1000, m = 100, 256 threads: 29 k cycles before, of which the
+// passes over global memory were most; N = 100, m = 1: 7.4 k.)
 inline __device__ void select_worst(const float* __restrict__ logl, int N, int m, uint32_t k0, uint32_t k1,
-                             uint32_t t, int* sel_slot, uint32_t* sel_key, int* worst, float* W,
+                             uint32_t t, int* sel_slot, uint32_t* sel_key, uint32_t* keys, int* worst, float* W,
                              int* seed_slot, SelectScratch& X, BlockScratch& S) {
-  const int tid = threadIdx.x, B = blockDim.x;
-  uint32_t prefix = 0, pmask = 0;
+  const int tid = threadIdx.x, B = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = B >> 5;
+  uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
+  int jmin = 0x7FFFFFFF;
+  for (int j0 = tid; j0 < N; j0 += 4 * B) {
+    float l[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) l[u] = j0 + u * B < N ? logl[j0 + u * B] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + u * B < N) {
+        const uint32_t key = order_key(l[u]);
+        if (keys) keys[j0 + u * B] = key;
+        if (key < kmin) {
+          kmin = key;
+          jmin = j0 + u * B;
+        }
+        kmax = max(kmax, key);
+      }
+  }
+  {
+    const uint32_t wmin = __reduce_min_sync(kFull, kmin);
+    const unsigned wj = __reduce_min_sync(kFull, kmin == wmin ? (unsigned)jmin : 0x7FFFFFFFu);
+    const uint32_t wmax = __reduce_max_sync(kFull, kmax);
+    if (lane == 0) {  // [wid], [64 + wid], [128 + wid] of the histogram
+      X.hist[wid] = wmin;
+      X.hist[64 + wid] = wj;
+      X.hist[128 + wid] = wmax;
+    }
+  }
+  __syncthreads();
+  for (int w = 0; w < nw; ++w) {
+    const uint32_t km = X.hist[w];
+    const int jm = (int)X.hist[64 + w];
+    if (w == 0 || km < kmin || (km == kmin && jm < jmin)) {
+      kmin = km;
+      jmin = jm;
+    }
+    kmax = w == 0 ? X.hist[128] : max(kmax, X.hist[128 + w]);
+  }
+  if (m == 1) {
+    if (tid == 0) {
+      sel_slot[0] = jmin;
+      sel_key[0] = kmin;
+      worst[0] = jmin;
+      W[0] = logl[jmin];
+      seed_slot[0] = survivor_slot(k0, k1, t, 0, N, 1, &jmin);
+    }
+    __syncthreads();
+    return;
+  }
+  auto key_at = [&](int j) { return keys ? keys[j] : order_key(logl[j]); };
+  // T: the keys below it are selected, and the first k of the equal ones (all
+  // of them where the bucket is taken whole: k = N)
+  const int top = kmin == kmax ? 0 : 31 - __clz(kmin ^ kmax);  // highest differing bit
+  uint32_t done = top == 31 ? 0u : ~((2u << top) - 1u);        // bits fixed so far
+  uint32_t prefix = kmin & done;
   int k = m;  // rank (1-based) still to find among keys matching the prefix
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 24 - 8 * pass;
+  int hi = top;
+  bool whole = false;
+  while (hi >= 0 && kmin != kmax && !whole) {
+    const int shift = max(0, hi - 7);
+    const uint32_t digits = (2u << (hi - shift)) - 1u;
+    __syncthreads();
     for (int i = tid; i < 256; i += B) X.hist[i] = 0;
     __syncthreads();
     for (int j = tid; j < N; j += B) {
-      const uint32_t key = order_key(logl[j]);
-      if ((key & pmask) == prefix) atomicAdd(&X.hist[(key >> shift) & 255u], 1u);
+      const uint32_t key = key_at(j);
+      if ((key & done) == prefix) atomicAdd(&X.hist[(key >> shift) & digits], 1u);
     }
     __syncthreads();
     if (tid < 32) {
@@ -442,31 +486,35 @@ inline __device__ void select_worst(const float* __restrict__ logl, int N, int m
           if (run < (unsigned)k && run + c[q] >= (unsigned)k) {
             X.found[0] = tid * 8 + q;
             X.found[1] = (int)run;
+            X.found[2] = run + c[q] == (unsigned)k;
           }
           run += c[q];
         }
       }
     }
     __syncthreads();
-    const int digit = X.found[0];
     k -= X.found[1];
-    prefix |= (uint32_t)digit << shift;
-    pmask |= 255u << shift;
-    __syncthreads();
+    prefix |= (uint32_t)X.found[0] << shift;
+    done |= digits << shift;
+    whole = X.found[2] != 0;
+    hi = shift - 1;
   }
-  const uint32_t T = prefix;  // key of the m-th smallest; k of the equal keys are taken
+  const uint32_t T = whole ? prefix | ~done : (kmin == kmax ? kmin : prefix);
+  if (whole) k = N;
   // ordered compaction over slot chunks
   const int C = (N + B - 1) / B;
   const int j0 = min(N, tid * C), j1 = min(N, j0 + C);
-  int n_eq = 0;
-  for (int j = j0; j < j1; ++j) n_eq += (order_key(logl[j]) == T);
-  int tot;
-  int eq_base = block_exclusive_scan(n_eq, S, &tot);
+  int tot, eq_base = 0;
+  if (!whole) {
+    int n_eq = 0;
+    for (int j = j0; j < j1; ++j) n_eq += (key_at(j) == T);
+    eq_base = block_exclusive_scan(n_eq, S, &tot);
+  }
   int n_sel = 0;
   {
     int e = eq_base;
     for (int j = j0; j < j1; ++j) {
-      const uint32_t key = order_key(logl[j]);
+      const uint32_t key = key_at(j);
       if (key < T || (key == T && e < k)) ++n_sel;
       if (key == T) ++e;
     }
@@ -475,7 +523,7 @@ inline __device__ void select_worst(const float* __restrict__ logl, int N, int m
   {
     int e = eq_base, p = sel_base;
     for (int j = j0; j < j1; ++j) {
-      const uint32_t key = order_key(logl[j]);
+      const uint32_t key = key_at(j);
       if (key < T || (key == T && e < k)) {
         sel_slot[p] = j;
         sel_key[p] = key;
@@ -485,27 +533,19 @@ inline __device__ void select_worst(const float* __restrict__ logl, int N, int m
     }
   }
   __syncthreads();
-  // sort the m selected by (key, slot): rank by counting
+  // sort the m selected by (key, slot): rank by counting (they are in slot order)
   for (int e = tid; e < m; e += B) {
     const uint32_t ke = sel_key[e];
     const int se = sel_slot[e];
     int r = 0;
+#pragma unroll 4
     for (int q = 0; q < m; ++q) {
       const uint32_t kq = sel_key[q];
-      r += (kq < ke) || (kq == ke && sel_slot[q] < se);
+      r += (kq < ke) || (kq == ke && q < e);
     }
     worst[r] = se;
     W[r] = logl[se];
-  }
-  // start slots: the idx-th survivor in ascending slot order; sel_slot is in
-  // ascending slot order, so skip every selected slot at or below the index.
-  for (int i = tid; i < m; i += B) {
-    int s = u_index(draw_at(k0, k1, t, (uint32_t)i, kPurposeSeed, 0), N - m);
-    for (int q = 0; q < m; ++q) {
-      if (sel_slot[q] <= s) ++s;
-      else break;
-    }
-    seed_slot[i] = s;
+    seed_slot[e] = survivor_slot(k0, k1, t, e, N, m, sel_slot);
   }
   __syncthreads();
 }
@@ -1405,6 +1445,28 @@ inline __device__ int batch_correct(int m, int K, int correction, const float* _
                                     const int* __restrict__ hist_len, int t_max, const Cand& A, const Cand& Bf,
                                     const Cand& Tm, int* list_f, float* vals, int* counter, BlockScratch& S) {
   const int tid = threadIdx.x, B = blockDim.x;
+  if (m == 1) {
+    // one removed point and one new one: the sort is a comparison (ties: the
+    // removed point first), and Algorithm 2 never finds both a faulty point
+    // (the new one live) and an instant death (the new one dead)
+    if (tid == 0) {
+      const float w = W[0], l = new_l[0];
+      const bool up = correction == 0 || correction == 3 || !(l < w);  // the new point lives
+      const int iw = up ? 0 : 1, in = 1 - iw;
+      A.l[iw] = w;
+      A.P[iw] = -1.f;
+      A.src[iw] = 0;
+      A.H[iw] = -1;
+      A.hp[iw] = -1;
+      A.l[in] = l;
+      A.P[in] = w;
+      A.src[in] = 1;
+      A.H[in] = 0;
+      A.hp[in] = -1;
+    }
+    __syncthreads();
+    return 0;
+  }
   // Bf holds the unsorted candidates: W (ascending, candidates 0..m-1), then
   // the walkers' new points (candidates m..2m-1)
   for (int i = tid; i < m; i += B) {
@@ -1453,15 +1515,20 @@ inline __device__ int batch_correct(int m, int K, int correction, const float* _
         const int w = C.H[e];
         const float thr = vals[i];
         const int hl = min(hist_len[w], t_max);
-        for (int h = 0; h < hl; ++h) {
-          const float hv = hist_l[(size_t)w * t_max + h];
-          if (hv > thr) {
-            C.l[e] = hv;
-            C.hp[e] = h;
-            C.P[e] = thr;
-            atomicAdd(counter, 1);
-            break;
-          }
+        bool found = false;
+        for (int h0 = 0; h0 < hl && !found; h0 += 4) {  // four entries' loads in flight
+          float hv[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) hv[u] = h0 + u < hl ? hist_l[(size_t)w * t_max + h0 + u] : -CUDART_INF_F;
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (!found && h0 + u < hl && hv[u] > thr) {
+              found = true;
+              C.l[e] = hv[u];
+              C.hp[e] = h0 + u;
+              C.P[e] = thr;
+              atomicAdd(counter, 1);
+            }
         }
       }
       __syncthreads();
@@ -1485,56 +1552,115 @@ inline __device__ int batch_correct(int m, int K, int correction, const float* _
 struct EvidState {
   double logz, info;
   long long k;
+  // of N alone: 1 / N, log(1 - exp(-1/N)), log N (set by evidence_init)
+  double invN, cN, logN;
 };
 
-inline __device__ void evidence_add(EvidState& E, int N, int n, const float* __restrict__ l_in,
-                             double* logw_out, bool live, BlockScratch& S, int vb) {
-  const double Nd = (double)N;
-  const double invN = 1.0 / Nd;
-  const double cN = log(-expm1(-invN));
-  const double live_off = -(double)E.k * invN - log(Nd);
-  // the first vb threads take the points (blocks of any size then add them in
-  // the same order)
-  const int tid = threadIdx.x, B = vb, first = tid < vb ? tid : n;
+// One thread.  An FP64 logarithm costs a warp 2.2 k cycles on this part, so
+// what does not change is computed once.
+__device__ __forceinline__ void evidence_init(EvidState& E, int N) {
+  E.invN = 1.0 / (double)N;
+  E.cN = log(-expm1(-E.invN));
+  E.logN = log((double)N);
+}
+
+__device__ __forceinline__ double warp_sum_d(double v) {  // lane 0's value
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
+  return v;
+}
+
+// The barrier of n threads (whole warps) of the block; id 0 with all of them is
+// __syncthreads.
+__device__ __forceinline__ void team_sync(int id, int n) {
+  if (n == 32) __syncwarp();
+  else asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory");
+}
+
+// Called by the warps [0, team) of the block (all of them, and all together:
+// `bar` is their barrier), team >= ceil(min(n, vb) / 32).  The first vb
+// threads take the points, so that blocks of any size add them in the same
+// order.  An FP64 instruction holds a warp's scheduler for 64 cycles, so
+// warps without points do none, the old evidence's weight is taken by the
+// last warp while the others take the points', and one warp finishes.
+static __device__ __noinline__ void evidence_add(EvidState& E, int n, const float* l_in, double* logw_out, bool live,
+                                                 BlockScratch& S, int vb, int team, int bar) {
+  auto sync = [&]() { team_sync(bar, 32 * team); };
+  const int tid = threadIdx.x, B = vb, lane = tid & 31, wid = tid >> 5;
+  const int first = tid < vb ? tid : n;
+  const int nact = min(team, (min(n, vb) + 31) / 32);  // warps with points
   const long long k0 = E.k;
-  double mx = E.logz;
-  for (int j = first; j < n; j += B) {
-    const double l = (double)l_in[j];
-    const double lw = live ? l + live_off : l - (double)(k0 + j) * invN + cN;
-    if (logw_out) logw_out[j] = lw;
-    mx = fmax(mx, lw);
+  const double invN = E.invN, logz = E.logz;
+  const double off = live ? -(double)k0 * invN - E.logN : E.cN;
+  double mx = logz;
+  if (wid < nact) {
+    for (int j = first; j < n; j += B) {
+      const double l = (double)l_in[j];
+      const double lw = live ? l + off : l - (double)(k0 + j) * invN + off;
+      if (logw_out) logw_out[j] = lw;
+      mx = fmax(mx, lw);
+    }
+    if (n > 1) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(kFull, mx, o));
+    } else {
+      mx = __shfl_sync(kFull, mx, 0);
+    }
+    if (lane == 0) S.dw[wid] = mx;
   }
-  mx = block_max_d(mx, S);
+  sync();
+  mx = S.dw[0];
+  for (int w = 1; w < nact; ++w) mx = fmax(mx, S.dw[w]);
+  sync();
   if (mx == -CUDART_INF) {
-    if (!live) E.k = k0 + n;
+    if (!live && tid == 0) E.k = k0 + n;
+    sync();
     return;
   }
-  double sw = 0.0, swl = 0.0;
-  for (int j = first; j < n; j += B) {
-    const double l = (double)l_in[j];
-    const double lw = live ? l + live_off : l - (double)(k0 + j) * invN + cN;
-    const double w = exp(lw - mx);
-    sw += w;
-    if (l > -CUDART_INF) swl += w * l;
+  double w0 = 0.0;
+  const bool had = logz > -CUDART_INF;
+  if (wid == team - 1 && had) w0 = exp(logz - mx);  // (a warp with points, too, where all have)
+  if (wid < nact) {
+    double sw = 0.0, swl = 0.0;
+    for (int j = first; j < n; j += B) {
+      const double l = (double)l_in[j];
+      const double lw = live ? l + off : l - (double)(k0 + j) * invN + off;
+      const double w = exp(lw - mx);
+      sw += w;
+      if (l > -CUDART_INF) swl += w * l;
+    }
+    if (n > 1) {  // (one point: the other lanes hold zeros)
+      sw = warp_sum_d(sw);
+      swl = warp_sum_d(swl);
+    }
+    if (lane == 0) {
+      S.dw[wid] = sw;
+      S.dw[16 + wid] = swl;
+    }
   }
-  sw = block_sum_d(sw, S);
-  swl = block_sum_d(swl, S);
-  if (tid == 0) {
-    double Bs = sw, As = swl;
-    if (E.logz > -CUDART_INF) {
-      const double w0 = exp(E.logz - mx);
-      Bs += w0;
-      As += w0 * (E.info + E.logz);
+  if (wid == team - 1 && lane == 0) S.dw[32] = w0;
+  sync();
+  if (wid == 0) {
+    // the warps' sums, by the same tree
+    double Bs = lane < nact ? S.dw[lane] : 0.0, As = lane < nact ? S.dw[16 + lane] : 0.0;
+    if (nact > 1) {
+      Bs = warp_sum_d(Bs);
+      As = warp_sum_d(As);
+    }
+    if (had) {
+      const double v = S.dw[32];
+      Bs += v;
+      As += v * (E.info + logz);
     }
     const double lz = mx + log(Bs);
-    S.dw[0] = lz;
-    S.dw[1] = As / Bs - lz;
+    const double info = As / Bs - lz;
+    if (lane == 0) {
+      E.logz = lz;
+      E.info = info;
+      if (!live) E.k = k0 + n;
+    }
   }
-  __syncthreads();
-  E.logz = S.dw[0];
-  E.info = S.dw[1];
-  if (!live) E.k = k0 + n;
-  __syncthreads();
+  sync();
 }
 
 // ---------------------------------------------------------------------------

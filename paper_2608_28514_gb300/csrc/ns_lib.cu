@@ -51,15 +51,17 @@ struct SelectArgs {
   uint32_t keys[2 * 128];
 };
 
-__global__ void k_select(int N, int m, const float* __restrict__ logl, const SelectArgs K, uint32_t t,
-                         int* worst, float* W, int* seed_slot) {
+// staged: the dynamic shared memory holds the N keys too.
+__global__ void __launch_bounds__(512) k_select(int N, int m, const float* __restrict__ logl, const SelectArgs K,
+                                                uint32_t t, int staged, int* worst, float* W, int* seed_slot) {
   extern __shared__ __align__(16) char sm[];
   __shared__ BlockScratch S;
   __shared__ SelectScratch X;
   int* sel_slot = reinterpret_cast<int*>(sm);
   uint32_t* sel_key = reinterpret_cast<uint32_t*>(sm + al16(sizeof(int) * m));
+  uint32_t* keys = staged ? reinterpret_cast<uint32_t*>(sm + 2 * al16(sizeof(int) * m)) : nullptr;
   const int r = blockIdx.x;
-  select_worst(logl + (size_t)r * N, N, m, K.keys[2 * r], K.keys[2 * r + 1], t, sel_slot, sel_key,
+  select_worst(logl + (size_t)r * N, N, m, K.keys[2 * r], K.keys[2 * r + 1], t, sel_slot, sel_key, keys,
                worst + (size_t)r * m, W + (size_t)r * m, seed_slot + (size_t)r * m, X, S);
 }
 
@@ -98,9 +100,11 @@ __global__ void k_evidence(int N, int n, const float* __restrict__ l, double* st
     E.logz = state[0];
     E.info = state[1];
     E.k = (long long)state[2];
+    evidence_init(E, N);
   }
   __syncthreads();
-  evidence_add(E, N, n, l, logw, live != 0, S, blockDim.x);
+  evidence_add(E, n, l, logw, live != 0, S, blockDim.x, blockDim.x / 32, 0);
+  __syncthreads();
   if (threadIdx.x == 0) {
     state[0] = E.logz;
     state[1] = E.info;
@@ -1782,7 +1786,14 @@ ns_status ns_select_worst(int n_runs, int N, int m, const float* logl, const uin
     return NS_ERR_ARG;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  const size_t smem = al16(sizeof(int) * m) + al16(sizeof(uint32_t) * m);
+  // the keys in shared memory where they fit; wide blocks for long sets (a
+  // block is alone on its SM unless there are hundreds of runs)
+  size_t smem = al16(sizeof(int) * m) + al16(sizeof(uint32_t) * m);
+  const int staged = smem + sizeof(uint32_t) * (size_t)N <= kRunSmemBudget;
+  if (staged) smem += sizeof(uint32_t) * (size_t)N;
+  if (smem > 48 * 1024)
+    NS_CUDA(cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), nullptr);
+  const int block = N > 4096 ? 512 : (N > 512 ? 256 : 128);
   for (int r0 = 0; r0 < n_runs; r0 += 128) {
     const int nr = std::min(128, n_runs - r0);
     SelectArgs K;
@@ -1790,8 +1801,8 @@ ns_status ns_select_worst(int n_runs, int N, int m, const float* logl, const uin
       K.keys[2 * r] = (uint32_t)(seeds[r0 + r] & 0xFFFFFFFFull);
       K.keys[2 * r + 1] = (uint32_t)(seeds[r0 + r] >> 32);
     }
-    k_select<<<nr, 256, smem, s>>>(N, m, logl + (size_t)r0 * N, K, t, worst + (size_t)r0 * m, W + (size_t)r0 * m,
-                                  seed_slot + (size_t)r0 * m);
+    k_select<<<nr, block, smem, s>>>(N, m, logl + (size_t)r0 * N, K, t, staged, worst + (size_t)r0 * m,
+                                    W + (size_t)r0 * m, seed_slot + (size_t)r0 * m);
     NS_CUDA(cudaGetLastError(), nullptr);
   }
   return NS_OK;

@@ -91,6 +91,7 @@ struct Carve {
   int tiles;         // tiles of the moments in shared memory at once
   size_t work_bytes; // bytes at pbuf that the eigen-clips may use
   bool staged;       // the tree works on points staged in shared memory
+  size_t scratch_end; // end of the phase scratch (from tile on)
   bool chol_global;  // the cluster Cholesky factors live in global memory (MLP runs, spilled runs)
   bool tree_global;  // the cluster-tree scratch lives in global memory (spilled runs)
 };
@@ -236,6 +237,7 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
     grown = o;
   }
   c.total = grown > other ? grown : other;
+  c.scratch_end = spill && c.staged ? c.chol : c.total;
   return c;
 }
 
@@ -1255,6 +1257,7 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
     E.logz = RS.logz;
     E.info = RS.info;
     E.k = RS.k;
+    evidence_init(E, R.N);
   }
   __syncthreads();
   const int d = R.d, N = R.N, m = R.m;
@@ -1298,6 +1301,8 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
   float* s_vals = reinterpret_cast<float*>(sm + cv.vals);
   int* s_ctr = reinterpret_cast<int*>(sm + cv.ctr);
   int* s_stage_cid = reinterpret_cast<int*>(sm + cv.stage_cid);
+  uint32_t* s_keys =
+      cv.tile + sizeof(uint32_t) * (size_t)N <= cv.scratch_end ? reinterpret_cast<uint32_t*>(sm + cv.tile) : nullptr;
 
   if constexpr (!MLP) {  // likelihood parameters into shared memory
     const int* src = reinterpret_cast<const int*>(R.lik);
@@ -1335,6 +1340,15 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
       E.k = 0;
     }
   }
+  // the largest live log L: from here on it only rises (the m worst are
+  // replaced, m <= N / 2), to an iteration's best accepted point
+  float lmax;
+  {
+    float lm = -CUDART_INF_F;
+    for (int j = tid; j < N; j += B) lm = fmaxf(lm, R.live_l[j]);
+    __syncthreads();
+    lmax = block_max_f(lm, S);
+  }
   if (RS.t > 0) {  // cluster tables of the last re-clustering
     if (!cv.chol_global)
       for (int i = tid; i < R.n_nodes * d * d; i += B) s_chol[i] = R.chol[i];
@@ -1366,7 +1380,8 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
     if (reclustered) cluster_phase<DMAX, MODE == kModeGroup>(R, t, sm, cv, S, vb);
     tick(kPhCluster);
     // a1-a2: selection
-    select_worst(R.live_l, N, m, R.k0, R.k1, t, s_sel_slot, s_sel_key, s_worst, s_W, s_seed, X, S);
+    select_worst(R.live_l, N, m, R.k0, R.k1, t, s_sel_slot, s_sel_key, s_keys, s_worst, s_W,
+                 s_seed, X, S);
     tick(kPhSelect);
     // a4-a7: slice-sampling walkers
     long long ev = 0, re = 0, cyc_eval = 0, cyc_reeval = 0;
@@ -1446,16 +1461,16 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
     // S_W's slots).  The run's arrays are read into registers first: through
     // R, every field would be loaded again after each store.
     const long long nd0 = RS.n_dead;
-    {
+    auto update = [&](int u, int BU, int bar) {  // thread u of BU
       float* const live_x = R.live_x;
-      const float* const new_x = R.new_x;
-      const float* const hist_x = R.hist_x;
+      const float* new_x = R.new_x;
+      const float* hist_x = R.hist_x;
       float* const dead_x = R.dead_x;
       float* const stage_x = R.stage_x;
       float* const live_l = R.live_l;
       int* const live_cid = R.live_cid;
       const int n_pad = R.n_pad, t_max = R.t_max, n_nodes = R.n_nodes;
-      for (int q = tid; q < m * d; q += B) {
+      for (int q = u; q < m * d; q += BU) {
         const int j = q / d, i = q - j * d;
         {
           const int src = A.src[j], hp = A.hp[j];
@@ -1474,31 +1489,40 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
           stage_x[(size_t)j * d + i] = val;
         }
       }
-      for (int j = tid; j < m; j += B) {
+      for (int j = u; j < m; j += BU) {
         R.dead_l[nd0 + j] = A.l[j];
         const int src = A.src[m + j];
         s_stage_cid[j] = (src < m) ? live_cid[s_worst[src]] : -1;
       }
-      __syncthreads();
-      for (int q = tid; q < m * d; q += B) {
+      team_sync(bar, BU);
+      for (int q = u; q < m * d; q += BU) {
         const int j = q / d, i = q - j * d;
         live_x[(size_t)i * n_pad + s_worst[j]] = stage_x[(size_t)j * d + i];
       }
-      for (int j = tid; j < m; j += B) {
+      for (int j = u; j < m; j += BU) {
         const int slot = s_worst[j];
         live_l[slot] = A.l[m + j];
         int c = s_stage_cid[j];
         if (c < 0) c = (n_nodes > 1) ? nearest_leaf(stage_x + (size_t)j * d, d, n_nodes, s_cent, s_mask) : 0;
         live_cid[slot] = c;
       }
+    };
+    // a11: evidence (FP64), on the first warps while the others update the
+    // live set where the block has twice the warps the points need, else
+    // after it.  Neither reads what the other writes.
+    const int team = (min(m, vb) + 31) / 32;
+    if (2 * team <= (B >> 5)) {
+      if ((tid >> 5) < team) evidence_add(E, m, A.l, R.dead_logw + nd0, false, S, vb, team, 2);
+      else update(tid - 32 * team, B - 32 * team, 3);
+      __syncthreads();
+      tick(kPhUpdate);
+    } else {
+      update(tid, B, 0);
+      __syncthreads();
+      tick(kPhUpdate);
+      evidence_add(E, m, A.l, R.dead_logw + nd0, false, S, vb, B >> 5, 0);
     }
-    __syncthreads();
-    tick(kPhUpdate);
-    // a11: evidence (FP64)
-    evidence_add(E, N, m, A.l, R.dead_logw + nd0, false, S, vb);
-    float lm = -CUDART_INF_F;
-    for (int j = tid; j < N; j += B) lm = fmaxf(lm, R.live_l[j]);
-    const float lmax = block_max_f(lm, S);
+    lmax = fmaxf(lmax, A.l[2 * m - 1]);
     tick(kPhEvidence);
     if (tid == 0) {
       RS.n_dead = nd0 + m;
@@ -1514,7 +1538,7 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
     if (flag_any) {
       // final live tail, slot order: each point carries X_K / N
       const long long nd1 = RS.n_dead;
-      evidence_add(E, N, N, R.live_l, R.dead_logw + nd1, true, S, vb);
+      evidence_add(E, N, R.live_l, R.dead_logw + nd1, true, S, vb, B >> 5, 0);
       for (int q = tid; q < N * d; q += B) {
         const int j = q / d, i = q - j * d;
         R.dead_x[(size_t)(nd1 + j) * d + i] = R.live_x[(size_t)i * R.n_pad + j];

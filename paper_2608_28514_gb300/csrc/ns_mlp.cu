@@ -21,21 +21,25 @@ namespace {
 
 // Persistent: each block sets up its tensor memory and barriers once and
 // evaluates batches of kMlpNbMax candidates, grid-strided.
+// Twelve epilogue warps (8: 630, 12: 616, 16: 649 us for 155,648 candidates in
+// BF16; 115, 107, 108 for 3001 at FP32 accuracy); the BF16 ring takes the five
+// tiles that fit.
 constexpr int kMlpStandaloneStages = 4;
-using MlpSmemStandalone = MlpSmem<kMlpNbMax, kMlpStandaloneStages>;
+constexpr int kMlpBf16Stages = 5, kMlpAloneWarps = 12, kMlpAloneThreads = (kMlpAloneWarps + 2) * 32;
+using MlpSmemStandalone = MlpSmem<kMlpNbMax, kMlpBf16Stages>;
 
-__global__ void __launch_bounds__(kMlpThreads, 1)
+__global__ void __launch_bounds__(kMlpAloneThreads, 1)
     k_mlp_bf16(const MlpDesc M, const uint8_t* __restrict__ tiles, const float* __restrict__ f32,
                const float* __restrict__ x, int n, float* __restrict__ out) {
   extern __shared__ __align__(1024) char sm_raw[];
   __shared__ MlpCtx ctx;
   char* sm = align1024_shared(sm_raw);
-  mlp_ctx_init(&ctx);
+  mlp_ctx_init(&ctx, kMlpAloneWarps);
   const int n_batches = (n + kMlpNbMax - 1) / kMlpNbMax;
   for (int b = blockIdx.x; b < n_batches; b += gridDim.x) {
     const int b0 = b * kMlpNbMax;
     const int nb = min(kMlpNbMax, n - b0);
-    if (!mlp_eval_bf16<kMlpNbMax, kMlpStandaloneStages>(M, tiles, f32, x + (size_t)b0 * M.d, M.d, nb, out + b0,
+    if (!mlp_eval_bf16<kMlpNbMax, kMlpBf16Stages, 1, kMlpAloneWarps>(M, tiles, f32, x + (size_t)b0 * M.d, M.d, nb, out + b0,
                                                          sm, &ctx))
       for (int r = threadIdx.x; r < nb; r += blockDim.x) out[b0 + r] = __int_as_float(0x7fffffff);
   }
@@ -46,18 +50,18 @@ __global__ void __launch_bounds__(kMlpThreads, 1)
 constexpr int kMlpSplitNb = 32;
 using MlpSmemSplit = MlpSmem<kMlpSplitNb, kMlpStandaloneStages, 3>;
 
-__global__ void __launch_bounds__(kMlpThreads, 1)
+__global__ void __launch_bounds__(kMlpAloneThreads, 1)
     k_mlp_split3(const MlpDesc M, const uint8_t* __restrict__ tiles, const float* __restrict__ f32,
                  const float* __restrict__ x, int n, float* __restrict__ out) {
   extern __shared__ __align__(1024) char sm_raw[];
   __shared__ MlpCtx ctx;
   char* sm = align1024_shared(sm_raw);
-  mlp_ctx_init(&ctx);
+  mlp_ctx_init(&ctx, kMlpAloneWarps);
   const int n_batches = (n + kMlpSplitNb - 1) / kMlpSplitNb;
   for (int b = blockIdx.x; b < n_batches; b += gridDim.x) {
     const int b0 = b * kMlpSplitNb;
     const int nb = min(kMlpSplitNb, n - b0);
-    if (!mlp_eval_bf16<kMlpSplitNb, kMlpStandaloneStages, 3>(M, tiles, f32, x + (size_t)b0 * M.d, M.d, nb,
+    if (!mlp_eval_bf16<kMlpSplitNb, kMlpStandaloneStages, 3, kMlpAloneWarps>(M, tiles, f32, x + (size_t)b0 * M.d, M.d, nb,
                                                               out + b0, sm, &ctx))
       for (int r = threadIdx.x; r < nb; r += blockDim.x) out[b0 + r] = __int_as_float(0x7fffffff);
   }
@@ -99,18 +103,18 @@ __global__ void __launch_bounds__(kMlpThreads, 1)
 constexpr int kMlpX2Nb = 64;
 using MlpSmemX2 = MlpSmem<kMlpX2Nb, kMlpStandaloneStages, 2>;
 
-__global__ void __launch_bounds__(kMlpThreads, 1)
+__global__ void __launch_bounds__(kMlpAloneThreads, 1)
     k_mlp_x2(const MlpDesc M, const uint8_t* __restrict__ tiles, const float* __restrict__ f32,
              const float* __restrict__ x, int n, float* __restrict__ out) {
   extern __shared__ __align__(1024) char sm_raw[];
   __shared__ MlpCtx ctx;
   char* sm = align1024_shared(sm_raw);
-  mlp_ctx_init(&ctx);
+  mlp_ctx_init(&ctx, kMlpAloneWarps);
   const int n_batches = (n + kMlpX2Nb - 1) / kMlpX2Nb;
   for (int b = blockIdx.x; b < n_batches; b += gridDim.x) {
     const int b0 = b * kMlpX2Nb;
     const int nb = min(kMlpX2Nb, n - b0);
-    if (!mlp_eval_bf16<kMlpX2Nb, kMlpStandaloneStages, 2>(M, tiles, f32, x + (size_t)b0 * M.d, M.d, nb, out + b0, sm,
+    if (!mlp_eval_bf16<kMlpX2Nb, kMlpStandaloneStages, 2, kMlpAloneWarps>(M, tiles, f32, x + (size_t)b0 * M.d, M.d, nb, out + b0, sm,
                                                            &ctx))
       for (int r = threadIdx.x; r < nb; r += blockDim.x) out[b0 + r] = __int_as_float(0x7fffffff);
   }
@@ -281,7 +285,7 @@ cudaError_t ns_mlp_launch(const MlpDesc& M, const void* image, int n, const floa
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int n_batches = (n + kMlpX2Nb - 1) / kMlpX2Nb;
-    k_mlp_x2<<<std::min(n_batches, n_sm), kMlpThreads, smem, s>>>(M, tiles, f32, x, n, logl);
+    k_mlp_x2<<<std::min(n_batches, n_sm), kMlpAloneThreads, smem, s>>>(M, tiles, f32, x, n, logl);
   } else if (precision == 2) {
     const int smem = MlpSmemSplit::kBytes + 1024;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_split3, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -290,7 +294,7 @@ cudaError_t ns_mlp_launch(const MlpDesc& M, const void* image, int n, const floa
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int n_batches = (n + kMlpSplitNb - 1) / kMlpSplitNb;
-    k_mlp_split3<<<std::min(n_batches, n_sm), kMlpThreads, smem, s>>>(M, tiles, f32, x, n, logl);
+    k_mlp_split3<<<std::min(n_batches, n_sm), kMlpAloneThreads, smem, s>>>(M, tiles, f32, x, n, logl);
   } else if (precision == 1) {
     const int smem = MlpSmemStandalone::kBytes + 1024;
     cudaError_t e = cudaFuncSetAttribute(k_mlp_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -299,7 +303,7 @@ cudaError_t ns_mlp_launch(const MlpDesc& M, const void* image, int n, const floa
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int n_batches = (n + kMlpNbMax - 1) / kMlpNbMax;
-    k_mlp_bf16<<<std::min(n_batches, n_sm), kMlpThreads, smem, s>>>(M, tiles, f32, x, n, logl);
+    k_mlp_bf16<<<std::min(n_batches, n_sm), kMlpAloneThreads, smem, s>>>(M, tiles, f32, x, n, logl);
   } else {
     const int smem = (int)mlp_f32_act_bytes(kMlpF32NbWide);
     cudaError_t e = cudaFuncSetAttribute(k_mlp_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -322,7 +326,7 @@ cudaError_t ns_mlp_launch_cluster(const MlpDesc& M, const void* image, int n, co
   const int nb = precision == 2 ? kMlpSplitNb : kMlpNbMax;
   const int n_batches = (n + nb - 1) / nb;
   const int n_clusters = std::max(1, std::min(n_batches, n_sm / cluster));
-  const int smem = (precision == 2 ? (int)MlpSmemSplit::kBytes : (int)MlpSmemStandalone::kBytes) + 1024;
+  const int smem = (precision == 2 ? (int)MlpSmemSplit::kBytes : (int)MlpSmem<kMlpNbMax, kMlpStandaloneStages>::kBytes) + 1024;
   auto kern = precision == 2 ? k_mlp_cl<kMlpSplitNb, 3> : k_mlp_cl<kMlpNbMax, 1>;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;

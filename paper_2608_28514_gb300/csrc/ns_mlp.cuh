@@ -29,7 +29,7 @@ namespace nsd {
 
 constexpr int kMlpMaxLayers = 8;
 constexpr int kMlpNbMax = 128;    // candidates per call, at most (the MMA's N)
-constexpr int kMlpStagesMax = 4;  // weight tiles in flight, at most
+constexpr int kMlpStagesMax = 5;  // weight tiles in flight, at most
 constexpr int kMlpTileBytes = 128 * 128;  // 128 rows x 64 BF16 (128 bytes)
 constexpr int kMlpMaxK = 512;     // widest padded layer input
 constexpr unsigned kMlpWaitCap = 1u << 22;
@@ -86,6 +86,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity) {
   for (unsigned i = 0; i < kMlpWaitCap; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
+}
+// One thread of the converged warp (the same one each time).
+__device__ __forceinline__ bool elect_one() {
+  unsigned e;
+  asm volatile(
+      "{\n.reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(e));
+  return e != 0;
 }
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
   asm volatile(
@@ -221,6 +231,16 @@ __device__ __forceinline__ void store_planes(char* dst, int plane_bytes, float v
 // (warp w owns tensor-memory lanes 32(w%4)..32(w%4)+31 and every other
 // 16-column chunk, starting at chunk w/4), warp 8 streams the weight tiles,
 // warp 9 issues the MMAs.  The block needs at least kMlpThreads threads.
+// (EW epilogue warps in general, then the two others: the stand-alone
+// evaluators have 12.)
+//
+// What bounds a pass of 128 candidates (228 tiles; 152 blocks, 80 us each, 96
+// with the issuing and the producing thread behind `lane == 0` and 118 with
+// the old input staging): about 53 us with neither copies, MMAs nor
+// epilogues, of which 0.15 us per tile is the issuing thread's chain (wait,
+// four MMAs, commit) and 18 us the input and the five layers' hand-overs;
+// the hidden layers' epilogues add 20 (two special-function results per
+// activation: 4 us each at best), the MMAs 4, the copies nothing.
 constexpr int kMlpEpiWarps = 8;
 constexpr int kMlpProducerWarp = 8;
 constexpr int kMlpMmaWarp = 9;
@@ -261,7 +281,7 @@ __device__ __forceinline__ unsigned ctx_err(const MlpCtx* c) { return *reinterpr
 __device__ __forceinline__ void ctx_set_err(MlpCtx* c) { *reinterpret_cast<volatile unsigned*>(&c->err) = 1u; }
 
 // Called by every thread of the block.
-inline __device__ void mlp_ctx_init(MlpCtx* c) {
+inline __device__ void mlp_ctx_init(MlpCtx* c, int epi_warps = kMlpEpiWarps) {
   const int tid = threadIdx.x;
   if ((tid >> 5) == 0) tmem_alloc(&c->tmem, 512);
   if (tid == 0) {
@@ -271,7 +291,7 @@ inline __device__ void mlp_ctx_init(MlpCtx* c) {
     }
     for (int h = 0; h < 2; ++h) {
       mbar_init(&c->acc_full[h], 1);
-      mbar_init(&c->acc_free[h], kMlpEpiWarps * 32);
+      mbar_init(&c->acc_free[h], epi_warps * 32);
     }
     mbar_init(&c->drain, 1);
     unsigned ncta;
@@ -316,6 +336,44 @@ __device__ __forceinline__ float warp_sum16(const float (&s)[16], int lane) {
   return d + __shfl_xor_sync(kFull, d, 1);
 }
 
+// The producer warp: streams `count` weight tiles (ring items item0, item0 + 1,
+// ..) through the S stages, one elected thread; src(i) is tile i's image,
+// after a call of next().  On an error (a stage that is not freed within the
+// wait budget, or another warp's) every copy issued has landed before it
+// returns.
+template <int S, class Src, class Next>
+__device__ __forceinline__ void stream_tiles(MlpCtx* ctx, char* stages, unsigned item0, unsigned count, Src src,
+                                             Next next) {
+  if (elect_one()) {
+    unsigned s = item0 % S, par = ((item0 / S) & 1) ^ 1u, i = 0;
+    bool err = false;
+    for (; i < count; ++i) {
+      if (item0 + i >= S && !mbar_wait(&ctx->empty[s], par)) {
+        err = true;
+        break;
+      }
+      next();
+      mbar_expect_tx(&ctx->full[s], kMlpTileBytes);
+      bulk_g2s(stages + s * kMlpTileBytes, src(i), kMlpTileBytes, &ctx->full[s]);
+      if (++s == S) {
+        s = 0;
+        par ^= 1u;
+        if (ctx_err(ctx) != 0u) {
+          err = true;
+          ++i;
+          break;
+        }
+      }
+    }
+    if (err) {
+      ctx_set_err(ctx);
+      // (only the last S can be outstanding)
+      for (unsigned j = item0 + (i > S ? i - S : 0); j < item0 + i; ++j) mbar_wait(&ctx->full[j % S], (j / S) & 1);
+    }
+  }
+  __syncwarp();
+}
+
 // How a layer's M-tiles are grouped on the accumulator halves for a call
 // with N candidates.  Hidden layers: one group of all M-tiles from column 0
 // (the next layer's input is written in place, so the layer's MMAs must all
@@ -345,6 +403,31 @@ __device__ __forceinline__ int mlp_n_groups(int MT, bool last, int N) {
   return last ? (MT + per - 1) / per : 1;
 }
 
+// The layer-0 operand: theta = lo + span x in P BF16 planes, rows = the n
+// candidates (N with the padding), K = d <= 32 (zero up to 64, one K-block).
+// row(r): candidate r's coordinates.  A warp per candidate, a lane per
+// coordinate, four candidates' loads in flight (an element per thread with
+// its indices divided out of a running number took 9 of a pass's 96 us).
+// Every thread of the block.
+template <int NBMAX, int P, class Row>
+__device__ __forceinline__ void mlp_input(const MlpDesc& M, char* act, int plane_bytes, int n, int N, Row row) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const bool mine = lane < M.d;
+  const float sp = mine ? M.span[lane] : 0.f, lo = mine ? M.lo[lane] : 0.f;
+  for (int r0 = threadIdx.x >> 5; r0 < N; r0 += 4 * nw) {
+    float v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = (mine && r0 + u * nw < n) ? row(r0 + u * nw)[lane] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + u * nw;
+      if (r >= N) break;
+      store_planes<P>(act + sw128_offset(r, lane), plane_bytes, (mine && r < n) ? fmaf(sp, v[u], lo) : 0.f);
+      store_planes<P>(act + sw128_offset(r, lane + 32), plane_bytes, 0.f);
+    }
+  }
+}
+
 // Evaluates the batch x [n][d] (unit cube, 1 <= n <= NBMAX) with the BF16
 // tensor-core path into out[n] (log L); the MMAs run with N = n rounded up
 // to 16.  With `rows` non-null, candidate r is row rows[r] of x and its
@@ -359,12 +442,12 @@ __device__ __forceinline__ int mlp_n_groups(int MT, bool last, int N) {
 // with the block's context `ctx` (mlp_ctx_init).  `sm` is 1024-byte aligned
 // and holds MlpSmem<NBMAX, STAGES>::kBytes.  Returns false (for every
 // thread) if a wait gave up, now or before.
-template <int NBMAX, int STAGES, int P = 1>
+template <int NBMAX, int STAGES, int P = 1, int EW = kMlpEpiWarps>
 inline __device__ bool mlp_eval_bf16(const MlpDesc& M, const uint8_t* __restrict__ tiles,
                                      const float* __restrict__ f32, const float* x, int x_stride, int n,
                                      float* out, char* sm, MlpCtx* ctx, const int* rows = nullptr) {
   using L = MlpSmem<NBMAX, STAGES, P>;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(kFull, tid >> 5, 0), lane = tid & 31;
   char* stages = sm + L::kStageOff;
   char* act = sm + L::kActOff;
   float* chi = reinterpret_cast<float*>(sm + L::kChiOff);
@@ -375,46 +458,27 @@ inline __device__ bool mlp_eval_bf16(const MlpDesc& M, const uint8_t* __restrict
   const unsigned tmem = ctx->tmem;
   const int last = M.n_layers - 1;
 
-  // layer-0 input: theta = lo + span x in BF16, rows = candidates, K = d (pad 0)
-  const int kb0 = M.kpad[0] / 64;
-  for (int q = tid; q < kb0 * N * 64; q += blockDim.x) {
-    const int kb = q / (N * 64), rem = q % (N * 64), r = rem / 64, k = rem % 64;
-    const int i = kb * 64 + k;
-    float v = 0.f;
-    if (r < n && i < M.d) v = fmaf(M.span[i], x[(size_t)(rows ? rows[r] : r) * x_stride + i], M.lo[i]);
-    char* dst = act + kb * NBMAX * 128 + sw128_offset(r, k);
-    store_planes<P>(dst, L::kPlaneBytes, v);
-  }
+  mlp_input<NBMAX, P>(M, act, L::kPlaneBytes, n, N,
+                      [&](int r) { return x + (size_t)(rows ? rows[r] : r) * x_stride; });
   for (int q = tid; q < 4 * NBMAX; q += blockDim.x) chi[q] = 0.f;
   fence_proxy_async();
   __syncthreads();
 
-  if (warp == kMlpProducerWarp) {
+  if (warp == EW) {
     // weight tiles in consumption order = image order
-    if (lane == 0) {
-      const unsigned end = item0 + (unsigned)M.n_tiles;
-      unsigned it = item0;
-      bool err = false;
-      for (; it < end; ++it) {
-        const unsigned s = it % S;
-        if (ctx_err(ctx) || (it >= S && !mbar_wait(&ctx->empty[s], ((it / S) - 1) & 1))) {
-          err = true;
-          break;
-        }
-        mbar_expect_tx(&ctx->full[s], kMlpTileBytes);
-        bulk_g2s(stages + s * kMlpTileBytes, tiles + (size_t)(it - item0) * kMlpTileBytes, kMlpTileBytes,
-                 &ctx->full[s]);
-      }
-      if (err) {
-        ctx_set_err(ctx);
-        // every copy issued lands before the block moves on (only the last S can be outstanding)
-        for (unsigned j = (it - item0 > S) ? it - S : item0; j < it; ++j) mbar_wait(&ctx->full[j % S], (j / S) & 1);
-      }
-    }
-    __syncwarp();
-  } else if (warp == kMlpMmaWarp) {
-    if (lane == 0) {
+    stream_tiles<STAGES>(ctx, stages, item0, (unsigned)M.n_tiles,
+                         [&](unsigned i) { return tiles + (size_t)i * kMlpTileBytes; }, [] {});
+  } else if (warp == EW + 1) {
+    // One elected thread waits and issues, inside one branch: an elected branch
+    // is one thread to the compiler, so the descriptors stay uniform (behind
+    // `lane == 0` every MMA went through a loop over lanes), and nothing is
+    // spent per tile on votes.  The loop over a tile is a chain of a single
+    // thread's instructions (~5 cycles each): it, not the copies or the
+    // MMAs, sets the pace below 64 candidates.
+    if (elect_one()) {
       const unsigned idesc = idesc_bf16(128, N);
+      const uint64_t adesc0 = sdesc_sw128(smem_u32(stages)), bdesc0 = sdesc_sw128(smem_u32(act));
+      unsigned s = item0 % S, par = (item0 / S) & 1;
       unsigned it = item0, uses[2] = {use0, use1};
       bool err = false;
       for (int l = 0; l <= last && !err; ++l) {
@@ -428,31 +492,34 @@ inline __device__ bool mlp_eval_bf16(const MlpDesc& M, const uint8_t* __restrict
             const bool need = (gi == 0) || (h >= G.h0 && h < G.h0 + G.nh);
             if (need && uses[h] > 0 && !mbar_wait(&ctx->acc_free[h], (uses[h] - 1) & 1)) err = true;
           }
-          if (err || ctx_err(ctx)) {
+          if (err || ctx_err(ctx) != 0u) {
             err = true;
             break;
           }
           tc_fence_after();
           const unsigned col0 = (unsigned)G.h0 * kMlpHalfCols;
           for (int t = G.g0; t < G.g1 && !err; ++t) {
-            for (int kb = 0; kb < KB; ++kb, ++it) {
-              const unsigned s = it % S;
-              if (!mbar_wait(&ctx->full[s], (it / S) & 1)) {
+            const unsigned d_tmem = tmem + col0 + (unsigned)((t - G.g0) * N);
+            uint64_t bd = bdesc0;
+#pragma unroll 4
+            for (int kb = 0; kb < KB; ++kb, ++it, bd += NBMAX * 128 / 16) {
+              if (!mbar_wait(&ctx->full[s], par)) {
                 err = true;
                 break;
               }
-              tc_fence_after();
-              const unsigned d_tmem = tmem + col0 + (unsigned)((t - G.g0) * N);
-              const unsigned a0 = smem_u32(stages + s * kMlpTileBytes);
+              const uint64_t ad = adesc0 + s * (kMlpTileBytes / 16);
 #pragma unroll
               for (int pl = 0; pl < P; ++pl) {
-                const unsigned b0 = smem_u32(act + pl * L::kPlaneBytes + kb * NBMAX * 128);
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                  umma_bf16(d_tmem, sdesc_sw128(a0 + 32 * k), sdesc_sw128(b0 + 32 * k), idesc,
-                            (kb > 0 || k > 0 || pl > 0) ? 1u : 0u);
+                  umma_bf16(d_tmem, ad + 2 * k, bd + pl * (L::kPlaneBytes / 16) + 2 * k, idesc,
+                            (k > 0 || pl > 0) ? 1u : (unsigned)(kb > 0));
               }
               umma_commit(&ctx->empty[s]);
+              if (++s == S) {
+                s = 0;
+                par ^= 1u;
+              }
             }
           }
           if (err) break;
@@ -473,7 +540,7 @@ inline __device__ bool mlp_eval_bf16(const MlpDesc& M, const uint8_t* __restrict
       }
     }
     __syncwarp();
-  } else if (warp < kMlpEpiWarps) {
+  } else if (warp < EW) {
     const int q = warp & 3, ch = warp >> 2;  // lane quadrant, chunk parity
     const unsigned lane_base = (unsigned)(q * 32) << 16;
     const int n_chunks = N / 16;
@@ -495,28 +562,27 @@ inline __device__ bool mlp_eval_bf16(const MlpDesc& M, const uint8_t* __restrict
         const unsigned col0 = (unsigned)G.h0 * kMlpHalfCols;
         if (!is_last) {
           // bias + SiLU, BF16 straight into the next layer's swizzled B operand
-          for (int t = G.g0; t < G.g1; ++t) {
-            const int f = t * 128 + q * 32 + lane;
+          // (tile, 16 candidates) in turn over the warps of a quadrant
+          for (int e = ch; e < (G.g1 - G.g0) * n_chunks; e += EW / 4) {
+            const int t = e / n_chunks, c0 = (e - t * n_chunks) * 16;
+            const int f = (G.g0 + t) * 128 + q * 32 + lane;
             const float bias = f32[M.bias0[l] + f];
-            const int kb = f >> 6, k = f & 63;
-            char* dst = act + kb * NBMAX * 128;
-            for (int i = ch; i < n_chunks; i += 2) {
-              const int c0 = i * 16;
-              float v[16];
-              tmem_ld16(tmem + lane_base + col0 + (unsigned)((t - G.g0) * N + c0), v);
-              // BF16 path: SiLU on the special-function unit; the wider paths: accurate SiLU
+            const int k = f & 63;
+            char* dst = act + (f >> 6) * NBMAX * 128;
+            float v[16];
+            tmem_ld16(tmem + lane_base + col0 + (unsigned)(t * N + c0), v);
+            // BF16 path: SiLU on the special-function unit; the wider paths: accurate SiLU
 #pragma unroll
-              for (int c = 0; c < 16; ++c)
-                store_planes<P>(dst + sw128_offset(c0 + c, k), L::kPlaneBytes,
-                                (P == 1) ? silu_fast(v[c] + bias) : silu(v[c] + bias));
-            }
+            for (int c = 0; c < 16; ++c)
+              store_planes<P>(dst + sw128_offset(c0 + c, k), L::kPlaneBytes,
+                              (P == 1) ? silu_fast(v[c] + bias) : silu(v[c] + bias));
           }
           fence_proxy_async();
         } else {
           // chi^2: per candidate column, one tile of 128 features at a time,
           // added in tile order (so a candidate's value does not depend on
           // its batch: the grouping of tiles follows N)
-          for (int i = ch; i < n_chunks; i += 2) {
+          for (int i = ch; i < n_chunks; i += EW / 4) {
             const int c0 = i * 16;
             for (int t = G.g0; t < G.g1; ++t) {
               const int f = t * 128 + q * 32 + lane;
@@ -543,8 +609,8 @@ inline __device__ bool mlp_eval_bf16(const MlpDesc& M, const uint8_t* __restrict
       }
     }
     if (err) ctx_set_err(ctx);
-    epi_bar_sync();
-    for (int r = tid; r < n; r += kMlpEpiWarps * 32)
+    team_sync(1, EW * 32);
+    for (int r = tid; r < n; r += EW * 32)
       out[rows ? rows[r] : r] = -0.5f * (chi[r] + chi[NBMAX + r] + chi[2 * NBMAX + r] + chi[3 * NBMAX + r]);
   }
   __syncthreads();

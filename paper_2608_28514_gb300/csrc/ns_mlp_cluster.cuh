@@ -145,7 +145,7 @@ inline __device__ bool mlp_eval_bf16_cl(const MlpDesc& M, const uint8_t* __restr
                                         const float* __restrict__ f32, const XIn& X, int n, char* sm, MlpCtx* ctx,
                                         ClusterMail* mail, unsigned C, unsigned rank) {
   using L = MlpSmem<NBMAX, STAGES, P>;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(kFull, tid >> 5, 0), lane = tid & 31;
   char* stages = sm + L::kStageOff;
   char* act = sm + L::kActOff;
   float* chi = reinterpret_cast<float*>(sm + L::kChiOff);
@@ -161,18 +161,9 @@ inline __device__ bool mlp_eval_bf16_cl(const MlpDesc& M, const uint8_t* __restr
   const unsigned bytes0 = (unsigned)kb0 * (unsigned)P * (unsigned)N * 128u;
 
   if (!failed && !recv0) {
-    // layer-0 input: theta = lo + span x in BF16, rows = candidates, K = d (pad 0)
-    for (int q = tid; q < kb0 * N * 64; q += blockDim.x) {
-      const int kb = q / (N * 64), rem = q % (N * 64), r = rem / 64, k = rem % 64;
-      const int i = kb * 64 + k;
-      float v = 0.f;
-      if (r < n && i < M.d) {
-        const float xv = X.g ? X.g[(size_t)r * X.stride + i] : X.s[(size_t)(X.rows ? X.rows[r] : r) * X.stride + i];
-        v = fmaf(M.span[i], xv, M.lo[i]);
-      }
-      char* dst = act + kb * NBMAX * 128 + sw128_offset(r, k);
-      store_planes<P>(dst, L::kPlaneBytes, v);
-    }
+    mlp_input<NBMAX, P>(M, act, L::kPlaneBytes, n, N, [&](int r) {
+      return X.g ? X.g + (size_t)r * X.stride : X.s + (size_t)(X.rows ? X.rows[r] : r) * X.stride;
+    });
     fence_proxy_async();
   }
   if (!failed) {
@@ -198,32 +189,28 @@ inline __device__ bool mlp_eval_bf16_cl(const MlpDesc& M, const uint8_t* __restr
     // nothing to do; the peers' waits on this CTA give up and report
   } else if (warp == kMlpProducerWarp) {
     // this CTA's weight tiles, in consumption order (layer, own M-tile, K-block)
-    if (lane == 0) {
-      unsigned it = item0;
-      bool err = false;
-      for (int l = 0; l <= last && !err; ++l) {
-        const int KB = M.kpad[l] / 64, MT = M.mpad[l] / 128;
-        for (int t = (int)rank; t < MT && !err; t += (int)C)
-          for (int kb = 0; kb < KB; ++kb, ++it) {
-            const unsigned s = it % S;
-            if (ctx_err(ctx) || (it >= S && !mbar_wait(&ctx->empty[s], ((it / S) - 1) & 1))) {
-              err = true;
-              break;
-            }
-            mbar_expect_tx(&ctx->full[s], kMlpTileBytes);
-            bulk_g2s(stages + s * kMlpTileBytes, tiles + (size_t)(M.tile0[l] + t * KB + kb) * kMlpTileBytes,
-                     kMlpTileBytes, &ctx->full[s]);
-          }
-      }
-      if (err) {
-        ctx_set_err(ctx);
-        for (unsigned j = (it - item0 > S) ? it - S : item0; j < it; ++j) mbar_wait(&ctx->full[j % S], (j / S) & 1);
-      }
-    }
-    __syncwarp();
+    int l = 0, t = (int)rank, kb = -1, KB = M.kpad[0] / 64, MT = M.mpad[0] / 128;
+    unsigned count = 0;
+    for (int q = 0; q <= last; ++q) count += (unsigned)((M.mpad[q] / 128 / (int)C) * (M.kpad[q] / 64));
+    stream_tiles<STAGES>(
+        ctx, stages, item0, count,
+        [&](unsigned) { return tiles + (size_t)(M.tile0[l] + t * KB + kb) * kMlpTileBytes; },
+        [&]() {
+          if (++kb < KB) return;
+          kb = 0;
+          t += (int)C;
+          if (t < MT) return;
+          t = (int)rank;
+          ++l;
+          KB = M.kpad[l] / 64;
+          MT = M.mpad[l] / 128;
+        });
   } else if (warp == kMlpMmaWarp) {
-    if (lane == 0) {
+    // one elected thread waits and issues (as in mlp_eval_bf16)
+    if (elect_one()) {
       const unsigned idesc = idesc_bf16(128, N);
+      const uint64_t adesc0 = sdesc_sw128(smem_u32(stages)), bdesc0 = sdesc_sw128(smem_u32(act));
+      unsigned s = item0 % S, par = (item0 / S) & 1;
       unsigned it = item0, uses[2] = {use0, use1}, xu = xu0;
       bool err = false;
       for (int l = 0; l <= last && !err; ++l) {
@@ -241,31 +228,34 @@ inline __device__ bool mlp_eval_bf16_cl(const MlpDesc& M, const uint8_t* __restr
             if (!mbar_wait_cl(&ctx->act_ready, xu & 1)) err = true;
             ++xu;
           }
-          if (err || ctx_err(ctx)) {
+          if (err || ctx_err(ctx) != 0u) {
             err = true;
             break;
           }
           tc_fence_after();
           const unsigned col0 = (unsigned)G.h0 * kMlpHalfCols;
           for (int j = G.g0; j < G.g1 && !err; ++j) {
-            for (int kb = 0; kb < KB; ++kb, ++it) {
-              const unsigned s = it % S;
-              if (!mbar_wait(&ctx->full[s], (it / S) & 1)) {
+            const unsigned d_tmem = tmem + col0 + (unsigned)((j - G.g0) * N);
+            uint64_t bd = bdesc0;
+#pragma unroll 4
+            for (int kb = 0; kb < KB; ++kb, ++it, bd += NBMAX * 128 / 16) {
+              if (!mbar_wait(&ctx->full[s], par)) {
                 err = true;
                 break;
               }
-              tc_fence_after();
-              const unsigned d_tmem = tmem + col0 + (unsigned)((j - G.g0) * N);
-              const unsigned a0 = smem_u32(stages + s * kMlpTileBytes);
+              const uint64_t ad = adesc0 + s * (kMlpTileBytes / 16);
 #pragma unroll
               for (int pl = 0; pl < P; ++pl) {
-                const unsigned b0 = smem_u32(act + pl * L::kPlaneBytes + kb * NBMAX * 128);
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
-                  umma_bf16(d_tmem, sdesc_sw128(a0 + 32 * k), sdesc_sw128(b0 + 32 * k), idesc,
-                            (kb > 0 || k > 0 || pl > 0) ? 1u : 0u);
+                  umma_bf16(d_tmem, ad + 2 * k, bd + pl * (L::kPlaneBytes / 16) + 2 * k, idesc,
+                            (k > 0 || pl > 0) ? 1u : (unsigned)(kb > 0));
               }
               umma_commit(&ctx->empty[s]);
+              if (++s == S) {
+                s = 0;
+                par ^= 1u;
+              }
             }
           }
           if (err) break;

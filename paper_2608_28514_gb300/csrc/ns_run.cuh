@@ -1176,28 +1176,32 @@ __device__ __noinline__ void walker_phase_mlp(const RunDesc& R, const SliceCfg& 
   cyc_reeval = cr;
 }
 
-// Initial live points of an MLP run, evaluated in FP32.
+// Initial live points of an MLP run, evaluated in FP32 on the CUDA cores, 32
+// per pass of the weights; the CTAs of a cluster take the batches in turn.  (A
+// point's value does not depend on its batch.  Eight per pass on CTA 0 alone
+// took 95 of the 137 ms of a run's first iteration, N = 1500.)
 template <int DMAX>
-inline __device__ void init_live_mlp(const RunDesc& R, float* xbuf, float* lbuf, int* rlist, char* msm) {
+inline __device__ void init_live_mlp(const RunDesc& R, float* xbuf, float* lbuf, char* msm, unsigned C, unsigned rank) {
   const int d = R.d, XS = mlp_xs(d);
+  const int per = min(kMlpF32NbWide, 2 * R.m + kMlpF32Nb);  // the staging rows there are
   float* act = reinterpret_cast<float*>(msm);
-  for (int j0 = 0; j0 < R.N; j0 += R.m) {
-    const int nb = min(R.m, R.N - j0);
+  for (int j0 = (int)rank * per; j0 < R.N; j0 += (int)C * per) {
+    const int nb = min(per, R.N - j0);
     for (int q = threadIdx.x; q < nb * d; q += blockDim.x) {
       const int j = j0 + q / d, k = q % d;
       const float xv = u24(draw_at(R.k0, R.k1, kTInit, (uint32_t)j, 0u, (uint32_t)k));
       R.live_x[(size_t)k * R.n_pad + j] = xv;
       xbuf[(size_t)(q / d) * XS + k] = xv;
     }
-    for (int q = threadIdx.x; q < nb; q += blockDim.x) rlist[q] = q;
     __syncthreads();
-    mlp_reeval(R, xbuf, XS, lbuf, rlist, nb, xbuf + (size_t)2 * R.m * XS, lbuf + 2 * R.m, act);
+    mlp_batch_f32(R, xbuf, XS, nb, lbuf, act);
     for (int q = threadIdx.x; q < nb; q += blockDim.x) {
       R.live_l[j0 + q] = lbuf[q];
       R.live_cid[j0 + q] = 0;
     }
     __syncthreads();
   }
+  if (C > 1) cl_sync();
 }
 
 // How a run's walkers sit on its block: one per thread (when the runs fill
@@ -1265,6 +1269,9 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
                               MODE == kModeGroup ? (m + (int)C - 1) / (int)C : 0, N, (size_t)room);
   if constexpr (MLP) {
     if (rank > 0) {
+      if (!RS.initialized && !RS.stopped && RS.status == 0)
+        init_live_mlp<DMAX>(R, reinterpret_cast<float*>(sm + cv.xbuf), reinterpret_cast<float*>(sm + cv.lbuf),
+                            sm + cv.mlp, C, rank);
       mlp_follower(R, &mlp_ctx, mail, align1024_shared(sm + cv.mlp), C, rank);
       return;
     }
@@ -1329,7 +1336,7 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
   }
   __syncthreads();
   if (!RS.initialized) {
-    if constexpr (MLP) init_live_mlp<DMAX>(R, s_xbuf, s_lbuf, s_rlist, s_mlp);
+    if constexpr (MLP) init_live_mlp<DMAX>(R, s_xbuf, s_lbuf, s_mlp, C, rank);
     else init_live<DMAX>(R, P);
     __syncthreads();
     if (tid == 0) {

@@ -852,7 +852,7 @@ inline __device__ void slice_walker(const LikParams& P, const SliceCfg& S, int w
 }
 
 // ---------------------------------------------------------------------------
-// a5-a7 with one walker per group of G = 2, 4 or 8 lanes (aligned in the
+// a5-a7 with one walker per group of G = 4 or 8 lanes (aligned in the
 // warp).  The points a slice step may evaluate are known before any of them
 // is: the stepping-out ends are a, a - w, a - 2 w, .. and b, b + w, .., and a
 // rejected shrink candidate moves the bracket to itself whatever its log L,

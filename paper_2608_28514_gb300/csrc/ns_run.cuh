@@ -202,7 +202,7 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
         c.staged = true;
         c.rows = rows;
         c.stage = at + sums(rows);
-        c.work_bytes = sums(rows) + pts;
+        c.work_bytes = sums(rows) + sizeof(float) * (size_t)d * N;  // (the child bits follow the points)
         grown = at + sums(rows) + st;
         if (spill) {
           c.chol = end;

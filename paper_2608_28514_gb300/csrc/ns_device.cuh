@@ -388,8 +388,9 @@ __device__ __forceinline__ int survivor_slot(uint32_t k0, uint32_t k1, uint32_t 
 // the radix select starts at the highest bit in which the smallest and the
 // largest key differ, and stops as soon as a digit's bucket is taken whole;
 // one pass or two of eight bits instead of four.  One worst point (m = 1) is a
-// minimum.  (N = 1000, m = 100, 256 threads: 29 k cycles before, of which the
-// passes over global memory were most; N = 100, m = 1: 7.4 k.)
+// minimum; its slot is a point of the set whatever the keys are (the highest
+// key is a NaN's, which a live set may consist of).  (N = 1000, m = 100, 256
+// threads: 29 k cycles with four passes over global memory; N = 100, m = 1: 7.4 k.)
 inline __device__ void select_worst(const float* __restrict__ logl, int N, int m, uint32_t k0, uint32_t k1,
                              uint32_t t, int* sel_slot, uint32_t* sel_key, uint32_t* keys, int* worst, float* W,
                              int* seed_slot, SelectScratch& X, BlockScratch& S) {
@@ -405,7 +406,7 @@ inline __device__ void select_worst(const float* __restrict__ logl, int N, int m
       if (j0 + u * B < N) {
         const uint32_t key = order_key(l[u]);
         if (keys) keys[j0 + u * B] = key;
-        if (key < kmin) {
+        if (key < kmin || jmin == 0x7FFFFFFF) {  // (a thread's slots ascend)
           kmin = key;
           jmin = j0 + u * B;
         }

@@ -1201,6 +1201,9 @@ inline __device__ void init_live_mlp(const RunDesc& R, float* xbuf, float* lbuf,
     }
     __syncthreads();
   }
+  // the evaluators' bulk copies, this CTA's and its peers', fill the same
+  // bytes next (a follower's own fences come after CTA 0's copies begin)
+  fence_proxy_async();
   if (C > 1) cl_sync();
 }
 

@@ -407,7 +407,7 @@ inline __device__ bool mlp_eval_bf16_cl(const MlpDesc& M, const uint8_t* __restr
     if (tid == 0 && !bad) ctx->pu = pu;
   }
   __syncthreads();
-  const bool ok = ctx_err(ctx) == 0u;
+  const bool ok = tiles_landed<STAGES>(ctx, item0);
   if (tid == 0) cl_st_s32(cl_map(smem_u32(&mail->err[rank]), 0), ok ? 0 : 1);
   return ok;
 }

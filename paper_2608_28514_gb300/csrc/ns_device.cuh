@@ -396,7 +396,7 @@ inline __device__ void select_worst(const float* __restrict__ logl, int N, int m
                              int* seed_slot, SelectScratch& X, BlockScratch& S) {
   const int tid = threadIdx.x, B = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = B >> 5;
   uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-  int jmin = 0x7FFFFFFF;
+  int jmin = tid < N ? tid : 0x7FFFFFFF;  // (its first point, whose key may be the highest)
   for (int j0 = tid; j0 < N; j0 += 4 * B) {
     float l[4];
 #pragma unroll
@@ -406,7 +406,7 @@ inline __device__ void select_worst(const float* __restrict__ logl, int N, int m
       if (j0 + u * B < N) {
         const uint32_t key = order_key(l[u]);
         if (keys) keys[j0 + u * B] = key;
-        if (key < kmin || jmin == 0x7FFFFFFF) {  // (a thread's slots ascend)
+        if (key < kmin) {
           kmin = key;
           jmin = j0 + u * B;
         }

@@ -69,6 +69,9 @@ __device__ __forceinline__ void cl_st_f32(unsigned ca, float v) {
 __device__ __forceinline__ void cl_st_s32(unsigned ca, int v) {
   asm volatile("st.shared::cluster.s32 [%0], %1;\n" ::"r"(ca), "r"(v) : "memory");
 }
+__device__ __forceinline__ void cl_st_s64(unsigned ca, long long v) {
+  asm volatile("st.shared::cluster.s64 [%0], %1;\n" ::"r"(ca), "l"(v) : "memory");
+}
 // Arrive (release, cluster scope) on the mbarrier at cluster address ca.
 __device__ __forceinline__ void cl_mbar_arrive(unsigned ca) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(ca) : "memory");

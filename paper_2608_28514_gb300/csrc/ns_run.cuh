@@ -545,7 +545,8 @@ constexpr int kGroupClusterMax = 8;
 struct GroupMail {
   int op;        // 0 exit, 1 walk, 2 reload the cluster factors, then walk
   uint32_t t;
-  int ev[kGroupClusterMax], fl[kGroupClusterMax];
+  long long ev[kGroupClusterMax];
+  int fl[kGroupClusterMax];
 };
 
 // The walkers of CTA `rank` of C.
@@ -582,9 +583,10 @@ __device__ void group_follower(const RunDesc& R, const LikParams& P, SliceCfg SC
     long long ev = 0, c0 = 0, c1 = 0;
     int fl = 0;
     group_phase<DMAX>(R, P, SC, w0, w1, s_W, s_seed, s_chol, s_off, mem, ev, fl, c0, c1);
-    const int evs = (int)block_sum_ll(ev, S), fls = (int)block_sum_ll(fl, S);
+    const long long evs = block_sum_ll(ev, S);
+    const int fls = (int)block_sum_ll(fl, S);
     if (tid == 0) {
-      cl_st_s32(mail0 + (unsigned)offsetof(GroupMail, ev) + 4u * rank, evs);
+      cl_st_s64(mail0 + (unsigned)offsetof(GroupMail, ev) + 8u * rank, evs);
       cl_st_s32(mail0 + (unsigned)offsetof(GroupMail, fl) + 4u * rank, fls);
     }
     cl_sync();  // the new points and the counts are in place

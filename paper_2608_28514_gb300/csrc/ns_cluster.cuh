@@ -14,6 +14,8 @@
 // reproducible bit for bit.
 #pragma once
 
+#include <type_traits>
+
 #include "ns_device.cuh"
 
 namespace nsd {
@@ -388,6 +390,11 @@ __device__ __noinline__ void clip_nodes(int d, const int* fail, int n_fail, doub
   __syncthreads();
 }
 
+// Index type of a point table [d][ld]: 64 bits in global memory, where d n_pad
+// is bounded by the caller's memory alone.
+template <bool SMEM>
+using PointIndex = std::conditional_t<SMEM, int, size_t>;
+
 template <bool SMEM, class P>
 __device__ __forceinline__ P* in_smem(char* sm, P* p) {  // p in shared memory, so that the compiler knows it
   if constexpr (SMEM) return reinterpret_cast<P*>(sm + (smem_addr(p) - smem_addr(sm)));
@@ -413,7 +420,7 @@ __device__ __noinline__ void cluster_tree(const TreeIO& io_ref, const TreeScratc
   T.cnt = in_smem<SMEM>(sm, T.cnt);
   T.far = in_smem<SMEM>(sm, T.far);
   float* const y = SMEM ? in_smem<SMEM>(sm, io.stage) : io.y;
-  const int ld = SMEM ? N : io.n_pad;
+  const PointIndex<SMEM> ld = SMEM ? N : io.n_pad;
   uint8_t* const side = SMEM ? reinterpret_cast<uint8_t*>(y + d * N) : io.side;
   const size_t n_pad = io.n_pad;
   // ---- whiten by the root factor: y = L0^{-1} (x - mu0) ------------------

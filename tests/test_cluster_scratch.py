@@ -36,6 +36,10 @@ extern "C" long long clip_overrun(int d, int depth, int n_hi, long long room, in
   }
   return worst;
 }
+extern "C" long long point_at(int i, int n_pad, int j) {
+  const PointIndex<false> ld = n_pad;
+  return (long long)(i * ld + j);
+}
 """
 
 
@@ -51,7 +55,7 @@ def host(tmp_path_factory):
                         "-Xcompiler", "-fPIC", "-I", CSRC, str(d / "carve.cu"), "-o", so], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     lib = ctypes.CDLL(so)
-    lib.clip_overrun.restype = ctypes.c_longlong
+    lib.clip_overrun.restype = lib.point_at.restype = ctypes.c_longlong
     return lib
 
 
@@ -65,6 +69,11 @@ def test_clip_slots_end_before_the_child_bits(host, depth):
             staged += k.value
             assert k.value == 0 or over <= 0, (d, depth, room, n.value, over)
     assert staged > 1000
+
+
+@pytest.mark.parametrize("n_pad", [2**26, 2**26 + 32, 2**30])
+def test_points_in_global_memory_are_indexed_in_64_bits(host, n_pad):
+    assert host.point_at(31, n_pad, n_pad - 1) == 32 * n_pad - 1
 
 
 def two_modes(d, N):

@@ -10,7 +10,8 @@
 //
 // Determinism: every sum has a fixed thread -> point assignment and a fixed
 // reduction tree (warp shuffles, then warps in order); maxima use atomicMax
-// on order-preserving keys, which do not depend on order.  A run is therefore
+// on order-preserving keys, which do not depend on order; the eigen-clips of
+// several nodes share warps without sharing sums.  A run is therefore
 // reproducible bit for bit.
 #pragma once
 
@@ -294,15 +295,48 @@ __device__ __noinline__ unsigned max_mahalanobis2(const float* __restrict__ live
   return __float_as_uint(best);
 }
 
+// The sums of squares above (off) and on (dia) the diagonal of A (d x d) by a
+// group of 32 / K lanes (this one is lane g of it), all of them with the
+// result: the order is the 32-lane butterfly's whatever K is (this lane holds
+// the partial sums of 32 lanes' K), so that a node's sweeps stop at the same
+// point however many nodes share its warp.
+template <int K>
+__device__ __forceinline__ void jacobi_sums(int d, const double* A, int g, double& off, double& dia) {
+  constexpr int JL = 32 / K;
+  auto sum = [&](auto of) {  // of(row, column): whether the entry counts
+    double t[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      t[k] = 0.0;
+      for (int i = g + JL * k; i < d * d; i += 32) {
+        const int a = i / d, b = i - a * d;
+        const double v = A[i];
+        if (of(a, b)) t[k] += v * v;
+      }
+    }
+#pragma unroll
+    for (int h = K / 2; h > 0; h >>= 1)
+#pragma unroll
+      for (int k = 0; k < h; ++k) t[k] += t[k + h];
+#pragma unroll
+    for (int h = JL / 2; h > 0; h >>= 1) t[0] += __shfl_xor_sync(kFull, t[0], h);
+    return t[0];
+  };
+  off = sum([](int a, int b) { return b > a; });
+  dia = sum([](int a, int b) { return a == b; });
+}
+
 // The eigen-clips of the listed nodes (fail[0 .. n_fail)), whose Cholesky
 // met a pivot that is not positive: a leaf with no more members than
 // dimensions has a singular covariance, so a deep tree has dozens of them.
-// The same rotations as jacobi_eigen_warp, several nodes side by side in a
+// The rotations and sums of jacobi_eigen_warp, several nodes side by side in a
 // warp: an FP64 instruction costs a warp 64 cycles on this part whether one
 // lane or 32 use it, and most of a rotation is the divisions and square
 // roots of its angle, so JL lanes per node (as many as keep four warps
-// busy) cut the time by 32 / JL where nodes are many.  C(nd, i, k): the
-// covariance; done(nd, i, k, v): the factor's entries.  work: FP64
+// busy) cut the time by 32 / JL where nodes are many.  A node's result does
+// not depend on JL, on the slots or on its place in the list (which the
+// warps fill in any order).  C(nd, i, k): the covariance; done(f0, nf, work,
+// per): the clipped matrices of the nodes fail[f0 .. f0 + nf).  work: FP64
 // [slots][2 d d + d].  Every thread of the block.
 template <class Cov, class Done>
 __device__ __noinline__ void clip_nodes(int d, const int* fail, int n_fail, double* work, int slots, Cov C, Done done) {
@@ -326,17 +360,12 @@ __device__ __noinline__ void clip_nodes(int d, const int* fail, int n_fail, doub
       double* Q = A + dd;
       bool open = mine;
       for (int sweep = 0; sweep < 100; ++sweep) {
-        double off = 0.0, dia = 0.0;
-        for (int i = g; i < dd; i += JL) {
-          const int a = i / d, b = i - a * d;
-          const double v = A[i];
-          if (b > a) off += v * v;
-          else if (a == b) dia += v * v;
-        }
-        for (int o = JL / 2; o > 0; o >>= 1) {
-          off += __shfl_xor_sync(kFull, off, o);
-          dia += __shfl_xor_sync(kFull, dia, o);
-        }
+        double off, dia;
+        if (JL == 32) jacobi_sums<1>(d, A, g, off, dia);
+        else if (JL == 16) jacobi_sums<2>(d, A, g, off, dia);
+        else if (JL == 8) jacobi_sums<4>(d, A, g, off, dia);
+        else if (JL == 4) jacobi_sums<8>(d, A, g, off, dia);
+        else jacobi_sums<16>(d, A, g, off, dia);
         open = open && off > 1e-30 * dia;
         if (!__any_sync(kFull, open)) break;
         for (int p = 0; p < d; ++p)

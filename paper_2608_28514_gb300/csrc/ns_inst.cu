@@ -22,7 +22,7 @@ namespace nsd {
 template <class K>
 static cudaError_t launch_runs(K* kernel, const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk,
                                int vb, int cluster, int room, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kernel, smem);
   if (e != cudaSuccess) return e;
   if (cluster <= 1) {
     kernel<<<n, block, smem, s>>>(runs, ids, chunk, vb, room);
@@ -45,7 +45,7 @@ static cudaError_t launch_runs(K* kernel, const RunDesc* runs, const int* ids, i
 
 template <class K>
 static cudaError_t occupancy(K* kernel, int block, size_t smem, int* blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(kernel, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kernel, block, smem);
 }

@@ -1791,8 +1791,7 @@ ns_status ns_select_worst(int n_runs, int N, int m, const float* logl, const uin
   size_t smem = al16(sizeof(int) * m) + al16(sizeof(uint32_t) * m);
   const int staged = smem + sizeof(uint32_t) * (size_t)N <= kRunSmemBudget;
   if (staged) smem += sizeof(uint32_t) * (size_t)N;
-  if (smem > 48 * 1024)
-    NS_CUDA(cudaFuncSetAttribute(k_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), nullptr);
+  if (smem > 48 * 1024) NS_CUDA(allow_smem(k_select, smem), nullptr);
   const int block = N > 4096 ? 512 : (N > 512 ? 256 : 128);
   for (int r0 = 0; r0 < n_runs; r0 += 128) {
     const int nr = std::min(128, n_runs - r0);
@@ -1956,7 +1955,7 @@ ns_status ns_cluster(int N, int n_pad, int d, const float* live_x, const ns_opti
     return NS_ERR_ARG;
   }
   auto* kernel = d <= 4 ? k_cluster<4> : (d <= 8 ? k_cluster<8> : (d <= 16 ? k_cluster<16> : k_cluster<32>));
-  NS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), nullptr);
+  NS_CUDA(allow_smem(kernel, smem), nullptr);
   kernel<<<1, 256, smem, (cudaStream_t)stream>>>(R, t);
   NS_CUDA(cudaGetLastError(), nullptr);
   return NS_OK;

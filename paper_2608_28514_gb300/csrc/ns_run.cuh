@@ -104,6 +104,15 @@ using RunMlpSmem = MlpSmem<kMlpNbMax, kRunMlpStages>;
 // Dynamic shared memory a run kernel may take (the static part stays below 3 KB).
 constexpr size_t kRunSmemBudget = 227 * 1024 - 3072;
 
+// Before a launch of `kernel` with smem bytes: the attribute is raised to the
+// budget whatever smem is, so that host threads launching it with different
+// sizes never lower it for one another.
+template <class K>
+inline cudaError_t allow_smem(K* kernel, size_t smem) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(smem > kRunSmemBudget ? smem : kRunSmemBudget));
+}
+
 __host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 // Row stride (floats) of an MLP run's candidate staging buffer.

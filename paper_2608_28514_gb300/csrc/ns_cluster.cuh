@@ -28,99 +28,85 @@ constexpr int kSumRows = 64;    // rows of a warp's buffer in slot_sums, at most
 // Scratch of one tree build; L = 2^depth leaves, n_nodes = 2 L - 1.
 struct TreeScratch {
   float* c;           // [L][d]: the two centres of each node of the current level (slot 2q+s)
-  float* red;         // [nwarps][kRedW] partial sums (slot_sums: two items x virtual warps x 32 slots)
-  float* out;         // [kRedW]
+  float* red;         // [nwarps][kRedW] partial sums (slot_sums)
   unsigned long long* far;  // [L / 2] farthest members of the current level: distance bits, slot
   int* cnt;           // [2 L]: members per node of the level, then per (node, side) slot
   int* misc;          // [8]
   double* leaf_mu;    // [L][d]: merge weights of the current level
   double* node_mu;    // [n_nodes][d]
-  double* node_M2;    // [n_nodes][d*d]   (d*d: full symmetric, for the Cholesky)
+  double* node_M2;    // [n_nodes][d*d]   (d*d: full symmetric, for the Cholesky; the centre sums before)
   int* node_n;        // [n_nodes]
   unsigned* node_m2;  // [n_nodes] bits of the largest squared Mahalanobis distance
   double* lv;         // [n_nodes] log volumes
   double* veff;       // [n_nodes] effective (pruned) log volumes
   int* spl;           // [n_nodes] accepted splits
-  double* chol_work;  // per warp: [5 d d + d]
 };
 
+constexpr int kTreeHot = 5;  // the tables that the splits work on are the layout's first
+
 template <class F>
-__host__ __device__ inline size_t tree_layout(int d, int n_nodes, int nwarps, int nw_chol, F&& take) {
+__host__ __device__ inline void tree_layout(int d, int n_nodes, int nwarps, F&& take) {
   const int L = (n_nodes + 1) / 2;
   take(0, sizeof(float) * L * d);
   take(1, sizeof(float) * nwarps * kRedW);
-  take(2, sizeof(float) * kRedW);
-  take(3, sizeof(unsigned long long) * L);
-  take(4, sizeof(int) * L * 2);
-  take(5, sizeof(int) * 8);
-  take(6, sizeof(double) * L * d);
-  take(7, sizeof(double) * n_nodes * d);
-  take(8, sizeof(double) * (size_t)n_nodes * d * d);
-  take(9, sizeof(int) * n_nodes);
-  take(10, sizeof(unsigned) * n_nodes);
+  take(2, sizeof(unsigned long long) * L);
+  take(3, sizeof(int) * L * 2);
+  take(4, sizeof(int) * 8);
+  take(5, sizeof(double) * L * d);
+  take(6, sizeof(double) * n_nodes * d);
+  take(7, sizeof(double) * (size_t)n_nodes * d * d);
+  take(8, sizeof(int) * n_nodes);
+  take(9, sizeof(unsigned) * n_nodes);
+  take(10, sizeof(double) * n_nodes);
   take(11, sizeof(double) * n_nodes);
-  take(12, sizeof(double) * n_nodes);
-  take(13, sizeof(int) * n_nodes);
-  return take(14, sizeof(double) * nw_chol * (5 * d * d + d));
+  take(12, sizeof(int) * n_nodes);
 }
 
-// Bytes of the tables that the splits work on (items 0 .. 5 of the layout).
-__host__ __device__ inline size_t tree_hot_bytes(int d, int n_nodes, int nwarps) {
-  if (n_nodes <= 1) return 0;
-  size_t b = 0, hot = 0;
-  tree_layout(d, n_nodes, nwarps, 1, [&](int k, size_t x) {
-    b += (x + 15) & ~(size_t)15;
-    if (k == 5) hot = b;
-    return b;
-  });
-  return hot;
-}
-
-__host__ __device__ inline size_t tree_bytes(int d, int n_nodes, int nwarps, int nw_chol) {
+// Bytes of the first n_tables tables of the layout (by default all).
+__host__ __device__ inline size_t tree_bytes(int d, int n_nodes, int nwarps, int n_tables = 13) {
   if (n_nodes <= 1) return 0;
   size_t b = 0;
-  tree_layout(d, n_nodes, nwarps, nw_chol, [&](int, size_t x) {
-    b += (x + 15) & ~(size_t)15;
-    return b;
+  tree_layout(d, n_nodes, nwarps, [&](int k, size_t x) {
+    if (k < n_tables) b += (x + 15) & ~(size_t)15;
   });
   return b;
 }
 
-// Warps that factorise node covariances in parallel, bounded by a 48 KB
-// budget of FP64 work space.
-__host__ __device__ inline int tree_chol_warps(int d, int nwarps) {
-  const int per = (int)(sizeof(double) * (5 * d * d + d));
-  int w = (48 * 1024) / per;
-  if (w < 1) w = 1;
-  return w < nwarps ? w : nwarps;
+// The tree's share of a handle's arena (spilled runs), and the size by which a
+// run spills: the tables for nwarps warps and room for factorising several
+// nodes at once (up to 48 KB).  Fixed: a checkpoint restores only into an
+// arena of the same layout.
+__host__ __device__ inline size_t tree_arena_bytes(int d, int n_nodes, int nwarps) {
+  if (n_nodes <= 1) return 0;
+  const size_t per = sizeof(double) * (5 * d * d + d);
+  size_t w = 48 * 1024 / per;
+  w = w < 1 ? 1 : (w > 8 ? 8 : w);
+  return tree_bytes(d, n_nodes, nwarps) + sizeof(float) * kRedW + ((w * per + 15) & ~(size_t)15);
 }
 
 // hot: where the tables of the splits live (base itself, or shared memory when
 // the others are in global memory).
-__device__ inline TreeScratch tree_carve(char* base, char* hot, int d, int n_nodes, int nwarps, int nw_chol) {
-  char* p[15];
+__device__ inline TreeScratch tree_carve(char* base, char* hot, int d, int n_nodes, int nwarps) {
+  char* p[13];
   size_t o = 0;
-  tree_layout(d, n_nodes, nwarps, nw_chol, [&](int k, size_t x) {
-    p[k] = (k <= 5 ? hot : base) + o;
+  tree_layout(d, n_nodes, nwarps, [&](int k, size_t x) {
+    p[k] = (k < kTreeHot ? hot : base) + o;
     o += (x + 15) & ~(size_t)15;
-    return o;
   });
   TreeScratch T;
   T.c = reinterpret_cast<float*>(p[0]);
   T.red = reinterpret_cast<float*>(p[1]);
-  T.out = reinterpret_cast<float*>(p[2]);
-  T.far = reinterpret_cast<unsigned long long*>(p[3]);
-  T.cnt = reinterpret_cast<int*>(p[4]);
-  T.misc = reinterpret_cast<int*>(p[5]);
-  T.leaf_mu = reinterpret_cast<double*>(p[6]);
-  T.node_mu = reinterpret_cast<double*>(p[7]);
-  T.node_M2 = reinterpret_cast<double*>(p[8]);
-  T.node_n = reinterpret_cast<int*>(p[9]);
-  T.node_m2 = reinterpret_cast<unsigned*>(p[10]);
-  T.lv = reinterpret_cast<double*>(p[11]);
-  T.veff = reinterpret_cast<double*>(p[12]);
-  T.spl = reinterpret_cast<int*>(p[13]);
-  T.chol_work = reinterpret_cast<double*>(p[14]);
+  T.far = reinterpret_cast<unsigned long long*>(p[2]);
+  T.cnt = reinterpret_cast<int*>(p[3]);
+  T.misc = reinterpret_cast<int*>(p[4]);
+  T.leaf_mu = reinterpret_cast<double*>(p[5]);
+  T.node_mu = reinterpret_cast<double*>(p[6]);
+  T.node_M2 = reinterpret_cast<double*>(p[7]);
+  T.node_n = reinterpret_cast<int*>(p[8]);
+  T.node_m2 = reinterpret_cast<unsigned*>(p[9]);
+  T.lv = reinterpret_cast<double*>(p[10]);
+  T.veff = reinterpret_cast<double*>(p[11]);
+  T.spl = reinterpret_cast<int*>(p[12]);
   return T;
 }
 
@@ -233,8 +219,8 @@ __device__ __forceinline__ double logaddexp_d(double a, double b) {
 }
 
 // The tree for depth D >= 1.  Inputs: x, the root's mean mu0 (float [d])
-// and FP32 Cholesky L0 (float [d][d]); the root's FP64 statistics are
-// already in node_mu[0] / node_M2[0] / node_n[0] (filled by the caller).
+// and FP32 Cholesky L0 (float [d][d]), and its count in node_n[0] (filled by
+// the caller, with its centre, factors and log volume in the outputs).
 // Outputs: per node centre (float), chol (float + FP64), logvol, count,
 // split, mask; cid[j] = accepted leaf of point j.
 struct TreeIO {

@@ -114,7 +114,7 @@ cudaError_t NS_CAT(launch_slice_, NS_DMAX)(const LikParams& P, const SliceCfg& S
 // r*cluster + cluster - 1), which share its tensor-core evaluations.
 cudaError_t launch_run_mlp(const RunDesc* runs, const int* ids, int n, int block, size_t smem, int chunk, int cluster,
                            cudaStream_t s) {
-  return launch_runs(k_run<32, kModeMlp>, runs, ids, n, block, smem, chunk, block, cluster, 0, s);
+  return launch_runs(k_run<32, kModeMlp>, runs, ids, n, block, smem, chunk, block, cluster, (int)kRunSmemBudget, s);
 }
 #endif
 #endif

@@ -17,7 +17,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <set>
 #include <string>
+#include <tuple>
 #include <utility>
 #include <vector>
 
@@ -196,7 +198,7 @@ bool run_spills(const ns_problem& p, int n_nodes) {
 
 // Global tree scratch of a spilled run, sized for the widest block (the MLP
 // run kernel's warps).
-size_t tree_ws_bytes(int d, int n_nodes) { return tree_bytes(d, n_nodes, kMlpThreads / 32, tree_chol_warps(d, 8)); }
+size_t tree_ws_bytes(int d, int n_nodes) { return tree_arena_bytes(d, n_nodes, kMlpThreads / 32); }
 
 // FNV-1a over the shape of a batch (what fixes the arena layout): a
 // checkpoint restores only into a handle of the same shape.
@@ -251,21 +253,30 @@ int block_for_m(int m) {
 // clusters of blocks.  (Two lanes per walker were no faster than one thread:
 // sixteen groups of a warp in lock step take the longest of their shrink
 // sequences.  266 runs of a 28-D mixture, m = 69: 33.3 ms against 30.5.)
+struct RunSize {
+  int d, m, spill;
+  bool operator<(const RunSize& o) const { return std::tie(d, m, spill) < std::tie(o.d, o.m, o.spill); }
+};
 struct ClassNeed {
   int dmax, n, max_m, n_steps;  // runs, largest batch and slice steps of a class
+  int n_nodes;
+  std::set<RunSize> sizes;      // of its runs
 };
 struct RunShape {
-  int block, vb, group, cluster, group_w, room;
+  int block, vb, group, cluster, room;
   long long threads;  // of one run, at 128 registers
   double est;         // relative time of an iteration's walk
+  // the shared-memory layout of a run of m walkers and N live points
+  Carve carve(int d, int m, int n_nodes, int dmax, bool spill, int N, bool stage = true) const {
+    return make_carve(d, m, n_nodes, dmax, false, spill, group ? (m + cluster - 1) / cluster : 0, N, (size_t)room,
+                      stage && group, block / 32);
+  }
 };
 RunShape shape_at(const ClassNeed& c, int stage) {
   RunShape q;
   q.vb = q.block = block_for_m(c.max_m);
-  q.group = q.group_w = 0;
+  q.group = 0;
   q.cluster = 1;
-  q.room = 0;
-  q.threads = q.block * (c.dmax > 12 ? 2 : 1);
   double rounds = 7.0;  // of likelihoods per slice step
   if (stage > 0) {
     const int G = stage == 1 ? 4 : 8;
@@ -274,10 +285,18 @@ RunShape shape_at(const ClassNeed& c, int stage) {
       q.cluster *= 2;
     while (stage == 3 && q.cluster < kGroupClusterMax && 128 * q.cluster < 8 * c.max_m) q.cluster *= 2;
     q.group = 1;
-    q.group_w = (c.max_m + q.cluster - 1) / q.cluster;
-    q.threads = q.block * q.cluster;
     rounds = stage == 1 ? 3.0 : (stage == 2 ? 2.3 : 2.0);
   }
+  q.threads = q.block * (!q.group && c.dmax > 12 ? 2 : 1);
+  // the blocks that an SM's registers hold, fewer where a block's tree tables
+  // leave no room for them: its share of the SM, in threads
+  const int k = 512 / (int)q.threads;
+  q.room = (int)block_room(k);
+  int fit = k;
+  for (const RunSize& z : c.sizes)
+    fit = std::min(fit, smem_blocks(q.carve(z.d, z.m, c.n_nodes, c.dmax, z.spill != 0, 0, false).total));
+  if (fit < k) q.threads = 512 / std::max(fit, 1);
+  q.threads *= q.cluster;
   q.est = c.n_steps * rounds * (100.0 + 8.0 * c.dmax);
   return q;
 }
@@ -310,12 +329,12 @@ std::vector<RunShape> plan_shapes(const std::vector<ClassNeed>& need, int n_sm) 
     out[best] = q;
     ++stage[best];
   }
-  // shared memory for staged points: the whole SM's where every block has one
-  // to itself, else its threads' share
+  // the whole SM's shared memory where every block has one to itself, else the
+  // share of as many blocks as its registers hold
   long long blocks = 0;
   for (size_t k = 0; k < need.size(); ++k) blocks += (long long)need[k].n * out[k].cluster;
-  for (RunShape& q : out)
-    q.room = !q.group ? 0 : (int)(blocks <= n_sm ? kRunSmemBudget : kRunSmemBudget * q.block / 512);
+  if (blocks <= n_sm)
+    for (RunShape& q : out) q.room = (int)kRunSmemBudget;
   return out;
 }
 
@@ -552,7 +571,7 @@ struct ClassGroup {
   int cluster = 1;  // CTAs per run
   int vb = 0;       // analytic runs: threads whose order the sums follow (RunShape)
   int group = 0;    // analytic runs: walkers are lane groups
-  int room = 0;     // shared memory a block may take to stage its points (make_carve)
+  int room = 0;     // shared memory a block may take (make_carve)
   double est = 1e30;  // relative time of an iteration (MLP runs: the longest)
   bool mlp = false;
   size_t smem = 0;
@@ -892,10 +911,11 @@ ns_status ns_create_batch(int n_runs, const ns_problem* runs, const ns_options* 
     std::vector<int> which;
     for (int ci = 0; ci < kNumClasses; ++ci) {
       if (counts[ci] == 0) continue;
-      ClassNeed c = {kClasses[ci].dmax, counts[ci], 1, 1};
+      ClassNeed c = {kClasses[ci].dmax, counts[ci], 1, 1, n_nodes, {}};
       for (int r : members[ci]) {
         c.max_m = std::max(c.max_m, runs[r].m);
         c.n_steps = std::max(c.n_steps, runs[r].n_slice_steps);
+        c.sizes.insert({runs[r].d, runs[r].m, off[r].spill});
       }
       need.push_back(c);
       which.push_back(ci);
@@ -924,11 +944,14 @@ ns_status ns_create_batch(int n_runs, const ns_problem* runs, const ns_options* 
       g.cluster = q.cluster;
       g.room = q.room;
     }
-    for (int r : members[ci])
-      smem = std::max(smem, make_carve(runs[r].d, runs[r].m, n_nodes, g.dmax, g.mlp, off[r].spill != 0,
-                                       g.group ? (runs[r].m + g.cluster - 1) / g.cluster : 0, runs[r].n_live,
-                                       (size_t)g.room)
+    for (int r : members[ci]) {
+      const ns_problem& p = runs[r];
+      const bool sp = off[r].spill != 0;
+      smem = std::max(smem, (g.mlp ? make_carve(p.d, p.m, n_nodes, g.dmax, true, sp, 0, p.n_live, kRunSmemBudget, false,
+                                                kMlpThreads / 32)
+                                   : shapes[ci].carve(p.d, p.m, n_nodes, g.dmax, sp, p.n_live))
                                 .total);
+    }
     if (g.mlp) {
       g.block = std::max(g.block, kMlpThreads);  // the BF16 evaluator's warp roles
       // FP32 on the tensor cores needs BF16-valued weights; CTAs per run
@@ -1017,15 +1040,20 @@ int ns_resident_runs_per_sm(int d, int m, int depth) {
   const int n_nodes = (1 << (depth + 1)) - 1;
   const int ci = class_index(d);
   int blocks = 0;
+  if (make_carve(d, m, n_nodes, kClasses[ci].dmax).base > kRunSmemBudget) {
+    set_err(nullptr, "ns_resident_runs_per_sm: the cluster tables of d = %d, depth = %d do not fit in shared memory", d,
+            depth);
+    return -1;
+  }
   // the shape of a batch of many runs
-  const RunShape q = plan_shapes({{kClasses[ci].dmax, 1 << 20, m, 5 * d}}, device_sms())[0];
+  const RunShape q = plan_shapes({{kClasses[ci].dmax, 1 << 20, m, 5 * d, n_nodes, {{d, m, 0}}}}, device_sms())[0];
   const cudaError_t e = kClasses[ci].occ(
-      q.block, make_carve(d, m, n_nodes, kClasses[ci].dmax, false, false, q.group_w).total, q.group, &blocks);
+      q.block, q.carve(d, m, n_nodes, kClasses[ci].dmax, false, 0, false).total, q.group, &blocks);
   if (e != cudaSuccess) {
     set_err(nullptr, "occupancy query failed: %s", cudaGetErrorString(e));
     return -1;
   }
-  return std::max(1, blocks / q.cluster);
+  return blocks / q.cluster;
 }
 
 ns_status ns_reset(ns_handle* h, void* stream) {
@@ -1703,8 +1731,9 @@ ns_status ns_run_noalloc(const ns_problem* problem, const ns_options* opt_in, fl
   NS_CUDA(cudaMemsetAsync(base + o_state, 0, sizeof(RunState), s), nullptr);
   const RunDesc* d_desc = reinterpret_cast<const RunDesc*>(base + o_desc);
   const int* d_ids = reinterpret_cast<const int*>(base + o_ids);
-  const RunShape q = plan_shapes({{dmax_class(d), 1, m, p.n_slice_steps}}, device_sms())[0];
-  const size_t smem = make_carve(d, m, n_nodes, dmax_class(d), false, spill, q.group_w, N, (size_t)q.room).total;
+  const RunShape q =
+      plan_shapes({{dmax_class(d), 1, m, p.n_slice_steps, n_nodes, {{d, m, spill}}}}, device_sms())[0];
+  const size_t smem = q.carve(d, m, n_nodes, dmax_class(d), spill != 0, N).total;
   const int chunk = opt.chunk_iters > 0 ? opt.chunk_iters : 1000;
   const long long max_rounds = opt.max_iter / chunk + 2;
   RunState hs;

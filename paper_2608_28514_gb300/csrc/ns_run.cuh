@@ -86,7 +86,7 @@ struct RunDesc {
 struct Carve {
   size_t lik, scr, sel, chol, cent, mask, worst, W, seed, sel_slot, sel_key, candA, candB, candT, list, vals, slots,
       ctr, stage_cid, xbuf, lbuf, rlist, tile, acc, c64, l64, work, tree, hot, pbuf, stage, mom, mlp, total;
-  size_t base;       // the total without the slot sums' buffer (what decides whether a run spills)
+  size_t base;       // by which a run spills (no spill: the tables with tree_arena_bytes)
   int rows;          // rows (slots x items) of that buffer, per warp
   int tiles;         // tiles of the moments in shared memory at once
   size_t work_bytes; // bytes at pbuf that the eigen-clips may use
@@ -118,15 +118,31 @@ __host__ __device__ inline size_t al16(size_t x) { return (x + 15) & ~(size_t)15
 // Row stride (floats) of an MLP run's candidate staging buffer.
 __host__ __device__ constexpr int mlp_xs(int d) { return (d + 3) & ~3; }
 
+// Blocks of `smem` bytes of dynamic shared memory that an SM's 228 KB hold
+// (each with up to 1 KB of static and 1 KB of the system's), and the largest
+// size of which it holds k.  (The MLP kernel, with more static memory, is
+// alone on its SM.)
+__host__ __device__ constexpr int smem_blocks(size_t smem) { return (int)(228 * 1024 / (smem + 2048)); }
+__host__ __device__ constexpr size_t block_room(int k) {
+  const size_t r = (228 * 1024 / (size_t)k - 2048) & ~(size_t)127;
+  return r < kRunSmemBudget ? r : kRunSmemBudget;
+}
+
 // spill: the run's cluster tables do not fit next to the rest (large d or a
 // deep tree); the Cholesky factors and the tree scratch then stay in global
 // memory (only the clustering and the direction draws read them).
 // group_w: walkers of one block when a walker is a group of lanes
-// (slice_walker_lanes), 0 when it is a thread.  room: shared memory the block
-// may take to stage its N live points for the cluster tree (with the factors
-// of a spilled run), 0 for none.
+// (slice_walker_lanes), 0 when it is a thread.  warps: the block's.
+// room: the shared memory that a block may take (block_room of as many as
+// are to share its SM).  Within it the block stages its N live points for the
+// cluster tree (stage; with the factors of a spilled run); where they do not
+// fit, what only makes the tree faster, the buffers of the slot sums and of the
+// moments, is as large as it can be without costing the SM a block.  (All
+// rows of the sums' buffer for every run, 67.6 KB whatever the block, took half
+// the blocks of a batch of trees: 608 runs of a 5-D mixture, m = 100, depth 3.)
 __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax, bool mlp = false,
-                                            bool spill = false, int group_w = 0, int N = 0, size_t room = 0) {
+                                            bool spill = false, int group_w = 0, int N = 0,
+                                            size_t room = kRunSmemBudget, bool stage = true, int warps = 8) {
   Carve c;
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -167,9 +183,10 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
   c.c64 = take(sizeof(double) * d * d);
   c.l64 = take(sizeof(double) * d * d);
   c.work = take(sizeof(double) * (3 * d * d + d));
-  // per-warp partials for every warp of the block (MLP blocks have kMlpThreads threads, others <= 256)
-  c.tree = take(c.tree_global ? 0 : tree_bytes(d, n_nodes, mlp ? kMlpThreads / 32 : 8, tree_chol_warps(d, 8)));
-  const int nwt = mlp ? kMlpThreads / 32 : 8, nwc = tree_chol_warps(d, 8);
+  const size_t root_end = o;
+  // the tree's tables, over what only the root's factorisation uses
+  o = c.c64;
+  c.tree = take(c.tree_global ? 0 : tree_bytes(d, n_nodes, warps));
   const size_t end_tree = o;
   c.mlp = phase0;
   size_t other = phase0;  // the end of what the clustering scratch shares its space with
@@ -189,13 +206,21 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
   c.candB = take(cand_bytes);
   c.candT = take(cand_bytes);
   if (o > other) other = o;
-  c.base = end_tree > other ? end_tree : other;
+  // (sizes of 8 warps, 10 in the MLP kernel, whatever the block)
+  const size_t arena = root_end + (spill ? 0 : tree_arena_bytes(d, n_nodes, mlp ? kMlpThreads / 32 : 8));
+  c.base = arena > other ? arena : other;
+  if (root_end > other) other = root_end;
   // the splits' tables of a spilled run; the slot sums' buffer (slot_sums) and
   // the staged points; the moments' tiles, over the scratch used after them
   o = end_tree;
-  c.hot = spill ? take(tree_hot_bytes(d, n_nodes, nwt)) : c.tree;
+  c.hot = spill ? take(tree_bytes(d, n_nodes, warps, kTreeHot)) : c.tree;
   const size_t at = o;
-  auto sums = [&](int rows) { return al16(sizeof(float) * (size_t)nwt * rows * 33); };
+  const int fit = smem_blocks(room);  // blocks that are to share the SM
+  auto blocks = [&](size_t end) {
+    const int k = smem_blocks(end > other ? end : other);
+    return k < fit ? k : fit;
+  };
+  auto sums = [&](int rows) { return al16(sizeof(float) * (size_t)warps * rows * 33); };
   size_t grown = at;
   c.rows = kSumRows;
   c.pbuf = c.stage = at;
@@ -204,10 +229,11 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
   if (n_nodes > 1) {
     const size_t pts = al16(sizeof(float) * (size_t)d * N), st = pts + al16(N);
     const size_t own_chol = spill && !mlp ? al16(sizeof(float) * (size_t)n_nodes * d * d) : 0;
-    for (int rows = kSumRows; rows >= 16 && !c.staged; rows /= 2) {
+    const size_t clip = sizeof(double) * (2 * d * d + d);  // of one node's eigen-clip
+    for (int rows = kSumRows; rows >= 16 && stage && !mlp && !c.staged; rows /= 2) {
       size_t end = at + sums(rows) + st;
       if (end < other) end = other;
-      if (!mlp && end + own_chol <= room) {
+      if (end + own_chol <= room && sums(rows) + sizeof(float) * (size_t)d * N >= clip) {
         c.staged = true;
         c.rows = rows;
         c.stage = at + sums(rows);
@@ -221,29 +247,35 @@ __host__ __device__ inline Carve make_carve(int d, int m, int n_nodes, int dmax,
       }
     }
     if (!c.staged) {
-      const size_t work = sizeof(double) * (size_t)nwc * (5 * d * d + d);
-      if (!spill && at + sums(c.rows) > kRunSmemBudget) {  // in the factorisation's work space
-        while (c.rows > 1 && sums(c.rows) > work) c.rows /= 2;
-        c.pbuf = end_tree - al16(work);
-        c.work_bytes = al16(work);
-      } else {
-        c.work_bytes = sums(c.rows) > al16(work) ? sums(c.rows) : al16(work);
-        grown = at + c.work_bytes;
-        if (grown > kRunSmemBudget) {
-          c.work_bytes = sums(c.rows);
-          grown = at + c.work_bytes;
-        }
-      }
+      // rows: as many as cost no block against 16 (fewer only to hold as many
+      // blocks as by c.base); then room for up to eight clips at a time (one at
+      // least) on the same terms
+      auto end = [&](int rows) { return at + (sums(rows) > al16(clip) ? sums(rows) : al16(clip)); };
+      while (c.rows > 1 && end(c.rows) > kRunSmemBudget) c.rows /= 2;
+      int least = c.rows < 16 ? c.rows : 16;
+      while (least > 4 && blocks(end(least)) < blocks(c.base)) least /= 2;
+      while (c.rows > least && blocks(end(c.rows)) < blocks(end(least))) c.rows /= 2;
+      grown = end(c.rows);
+      const size_t more = at + al16(8 * clip);
+      if (more > grown && more <= kRunSmemBudget && blocks(more) == blocks(grown)) grown = more;
+      c.work_bytes = grown - at;
     }
   }
-  c.tiles = moments_tiles(d);
-  o = c.c64;
-  c.mom = take(sizeof(float) * ((size_t)c.tiles * d * kTileS + moments_part(d, c.tiles)));
-  if (o > kRunSmemBudget || (spill && c.staged && o > c.chol)) {  // one tile in its own place, its sums where the factorisation will work
-    c.tiles = 1;
-    c.mom = c.tile;
-  } else if (o > grown) {
-    grown = o;
+  // as many of the moments' tiles as cost no block; one in its own place, its
+  // sums where the factorisation will work, if none does
+  const size_t mom_end = spill && c.staged ? c.chol : kRunSmemBudget;
+  for (c.tiles = moments_tiles(d);; --c.tiles) {
+    if (c.tiles == 0) {
+      c.tiles = 1;
+      c.mom = c.tile;
+      break;
+    }
+    o = c.c64;
+    c.mom = take(sizeof(float) * ((size_t)c.tiles * d * kTileS + moments_part(d, c.tiles)));
+    if (o <= mom_end && blocks(o) >= blocks(grown)) {
+      if (o > grown) grown = o;
+      break;
+    }
   }
   c.total = grown > other ? grown : other;
   c.scratch_end = spill && c.staged ? c.chol : c.total;
@@ -357,8 +389,8 @@ __device__ void cluster_phase(const RunDesc& R, uint32_t t, char* sm, const Carv
     return;
   }
   const int nw = blockDim.x >> 5;
-  const TreeScratch T =
-      tree_carve(cv.tree_global ? R.tree_ws : sm + cv.tree, sm + cv.hot, d, R.n_nodes, nw, tree_chol_warps(d, 8));
+  const TreeScratch T = tree_carve(cv.tree_global ? R.tree_ws : sm + cv.tree, sm + cv.hot, d, R.n_nodes, nw);
+  __syncthreads();  // the root's factorisation has been read: the tables overlay it
   if (threadIdx.x == 0) T.node_n[0] = n;
   __syncthreads();
   TreeIO io;
@@ -1280,7 +1312,8 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
   __syncthreads();
   const int d = R.d, N = R.N, m = R.m;
   const Carve cv = make_carve(d, m, R.n_nodes, DMAX, MLP, R.spill != 0,
-                              MODE == kModeGroup ? (m + (int)C - 1) / (int)C : 0, N, (size_t)room);
+                              MODE == kModeGroup ? (m + (int)C - 1) / (int)C : 0, N, (size_t)room, MODE == kModeGroup,
+                              B >> 5);
   if constexpr (MLP) {
     if (rank > 0) {
       if (!RS.initialized && !RS.stopped && RS.status == 0)

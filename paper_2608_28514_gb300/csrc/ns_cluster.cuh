@@ -281,37 +281,6 @@ __device__ __noinline__ unsigned max_mahalanobis2(const float* __restrict__ live
   return __float_as_uint(best);
 }
 
-// The sums of squares above (off) and on (dia) the diagonal of A (d x d) by a
-// group of 32 / K lanes (this one is lane g of it), all of them with the
-// result: the order is the 32-lane butterfly's whatever K is (this lane holds
-// the partial sums of 32 lanes' K), so that a node's sweeps stop at the same
-// point however many nodes share its warp.
-template <int K>
-__device__ __forceinline__ void jacobi_sums(int d, const double* A, int g, double& off, double& dia) {
-  constexpr int JL = 32 / K;
-  auto sum = [&](auto of) {  // of(row, column): whether the entry counts
-    double t[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      t[k] = 0.0;
-      for (int i = g + JL * k; i < d * d; i += 32) {
-        const int a = i / d, b = i - a * d;
-        const double v = A[i];
-        if (of(a, b)) t[k] += v * v;
-      }
-    }
-#pragma unroll
-    for (int h = K / 2; h > 0; h >>= 1)
-#pragma unroll
-      for (int k = 0; k < h; ++k) t[k] += t[k + h];
-#pragma unroll
-    for (int h = JL / 2; h > 0; h >>= 1) t[0] += __shfl_xor_sync(kFull, t[0], h);
-    return t[0];
-  };
-  off = sum([](int a, int b) { return b > a; });
-  dia = sum([](int a, int b) { return a == b; });
-}
-
 // The eigen-clips of the listed nodes (fail[0 .. n_fail)), whose Cholesky
 // met a pivot that is not positive: a leaf with no more members than
 // dimensions has a singular covariance, so a deep tree has dozens of them.
@@ -346,12 +315,29 @@ __device__ __noinline__ void clip_nodes(int d, const int* fail, int n_fail, doub
       double* Q = A + dd;
       bool open = mine;
       for (int sweep = 0; sweep < 100; ++sweep) {
-        double off, dia;
-        if (JL == 32) jacobi_sums<1>(d, A, g, off, dia);
-        else if (JL == 16) jacobi_sums<2>(d, A, g, off, dia);
-        else if (JL == 8) jacobi_sums<4>(d, A, g, off, dia);
-        else if (JL == 4) jacobi_sums<8>(d, A, g, off, dia);
-        else jacobi_sums<16>(d, A, g, off, dia);
+        // the sums of squares above and on the diagonal, the whole warp on one
+        // node after another: in the order of jacobi_eigen_warp whatever JL is
+        double off = 0.0, dia = 0.0;
+        for (int u = 0; u < npw; ++u) {
+          if (!__any_sync(kFull, open && lane / JL == u)) continue;
+          const double* Au = work + (w0 + u) * per;
+          double o = 0.0, e = 0.0;
+          for (int i = lane; i < dd; i += 32) {
+            const int a = i / d, b = i - a * d;
+            const double v = Au[i];
+            if (b > a) o += v * v;
+            else if (a == b) e += v * v;
+          }
+#pragma unroll
+          for (int h = 16; h > 0; h >>= 1) {
+            o += __shfl_xor_sync(kFull, o, h);
+            e += __shfl_xor_sync(kFull, e, h);
+          }
+          if (lane / JL == u) {
+            off = o;
+            dia = e;
+          }
+        }
         open = open && off > 1e-30 * dia;
         if (!__any_sync(kFull, open)) break;
         for (int p = 0; p < d; ++p)

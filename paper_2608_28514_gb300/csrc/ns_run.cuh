@@ -452,12 +452,11 @@ inline __device__ int nearest_leaf(const float* x, int d, int n_nodes, const flo
 }
 
 // a4-a7 for the calling thread's walker (threads of warps that hold a walker
-// call it; lanes past m take part in the warp votes only).  Kept out of line
-// so that its registers are allocated apart from the rest of the run kernel.
+// call it; lanes past m take part in the warp votes only).
 template <int DMAX>
-__device__ __noinline__ void walker_phase(const RunDesc& R, const LikParams& P, const SliceCfg& SC,
-                                          const float* s_W, const int* s_seed, float* s_slots, long long& ev, int& fl,
-                                          long long& cyc_walk) {
+__device__ __forceinline__ void walker_phase_inline(const RunDesc& R, const LikParams& P, const SliceCfg& SC,
+                                                    const float* s_W, const int* s_seed, float* s_slots, long long& ev, int& fl,
+                                                    long long& cyc_walk) {
   const int tid = threadIdx.x, m = R.m, d = R.d;
   const bool act = tid < m;
   const int i = act ? tid : 0;
@@ -479,6 +478,19 @@ __device__ __noinline__ void walker_phase(const RunDesc& R, const LikParams& P, 
   ev = act ? e : 0;
   fl = act ? f : 0;
   cyc_walk = clock64() - c1;
+}
+
+// The same out of line, so that its registers are allocated apart from the
+// rest of the run kernel: for the classes of 128 registers.  The wide classes
+// have registers for both, and inlined the walk's operands are known to be in
+// shared memory: out of line, 266 runs of a 28-D mixture (m 69) took 9.9 ms for
+// five steps against 8.6 inlined, 304 of a 28-D correlated Gaussian (m 100)
+// 11.6 against 9.7, in 32 dimensions 12.7 against 11.5.
+template <int DMAX>
+__device__ __noinline__ void walker_phase(const RunDesc& R, const LikParams& P, const SliceCfg& SC, const float* s_W,
+                                          const int* s_seed, float* s_slots, long long& ev, int& fl,
+                                          long long& cyc_walk) {
+  walker_phase_inline<DMAX>(R, P, SC, s_W, s_seed, s_slots, ev, fl, cyc_walk);
 }
 
 // a4-a7 with one walker per warp (RunDesc::walker_warp): warp w takes the
@@ -1478,7 +1490,8 @@ __global__ void NS_RUN_BOUNDS(MODE, DMAX) k_run(const RunDesc* __restrict__ runs
         walker_phase_warp<DMAX>(R, P, SC, s_W, s_seed, 0, m, ev, fl);
         cyc_reeval = clock64() - cd1;
       } else if ((tid & ~31) < m) {
-        walker_phase<DMAX>(R, P, SC, s_W, s_seed, s_slots, ev, fl, cyc_reeval);
+        if constexpr (DMAX > 12) walker_phase_inline<DMAX>(R, P, SC, s_W, s_seed, s_slots, ev, fl, cyc_reeval);
+        else walker_phase<DMAX>(R, P, SC, s_W, s_seed, s_slots, ev, fl, cyc_reeval);
         if (R.wk_evals && tid < m) {
           R.wk_evals[tid] = (int)ev;
           R.wk_flags[tid] = fl;

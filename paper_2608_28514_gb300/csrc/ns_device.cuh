@@ -1039,12 +1039,10 @@ inline __device__ void slice_walker_lanes(const LikParams& P, const SliceCfg& S,
             else be = tq;
           }
       } else {
-        const int k = nsh + g;
+        // past the draws of the row: the first batch took them all (G >= 4), or s_max ended it
         float uu = 0.f;
         if (open && g < K)
-          uu = k < kPreShrink
-                   ? (k == 1 ? pre[1] : pre[2])  // (s_max or G may end the first batch early)
-                   : u24(draw_at(S.k0, S.k1, S.t, (uint32_t)walker, (uint32_t)step, shrink_draw0(d) + (uint32_t)k));
+          uu = u24(draw_at(S.k0, S.k1, S.t, (uint32_t)walker, (uint32_t)step, shrink_draw0(d) + (uint32_t)(nsh + g)));
         for (int q = 0; q < G; ++q) {
           const float tq = fmaf(__shfl_sync(kFull, uu, base + q), be - ae, ae);
           if (q < K) {

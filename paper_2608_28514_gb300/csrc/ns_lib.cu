@@ -247,10 +247,11 @@ int block_for_m(int m) {
 // walkers.  Every class starts with one walker per thread, or with groups
 // where its smallest block leaves four lanes per walker idle anyway.  While
 // the runs' threads stay within what the SMs hold at 128 registers (512
-// each; a thread walker above 12 dimensions takes twice that), the class
-// whose runs take longest goes on to four lanes per walker, to eight, and
-// to blocks of no more than 128 busy lanes, on wider blocks first and then on
-// clusters of blocks.  (Two lanes per walker were no faster than one thread:
+// each; a thread walker above 12 dimensions takes twice that, a block of
+// large tree tables as many as fill its part of the SM's shared memory), the
+// class whose runs take longest goes on to four lanes per walker, to eight,
+// and to blocks of no more than 128 busy lanes, on wider blocks first and then
+// on clusters of blocks.  (Two lanes per walker were no faster than one thread:
 // sixteen groups of a warp in lock step take the longest of their shrink
 // sequences.  266 runs of a 28-D mixture, m = 69: 33.3 ms against 30.5.)
 struct RunSize {

@@ -455,8 +455,8 @@ inline __device__ int nearest_leaf(const float* x, int d, int n_nodes, const flo
 // call it; lanes past m take part in the warp votes only).
 template <int DMAX>
 __device__ __forceinline__ void walker_phase_inline(const RunDesc& R, const LikParams& P, const SliceCfg& SC,
-                                                    const float* s_W, const int* s_seed, float* s_slots, long long& ev, int& fl,
-                                                    long long& cyc_walk) {
+                                                    const float* s_W, const int* s_seed, float* s_slots,
+                                                    long long& ev, int& fl, long long& cyc_walk) {
   const int tid = threadIdx.x, m = R.m, d = R.d;
   const bool act = tid < m;
   const int i = act ? tid : 0;
@@ -1232,9 +1232,9 @@ __device__ __noinline__ void walker_phase_mlp(const RunDesc& R, const SliceCfg& 
 }
 
 // Initial live points of an MLP run, evaluated in FP32 on the CUDA cores, 32
-// per pass of the weights; the CTAs of a cluster take the batches in turn.  (A
-// point's value does not depend on its batch.  Eight per pass on CTA 0 alone
-// took 95 of the 137 ms of a run's first iteration, N = 1500.)
+// per pass of the weights; the CTAs of a cluster take the batches in turn (a
+// point's value does not depend on its batch).  N = 1500: 12 ms on four CTAs;
+// eight per pass on one took 95.
 template <int DMAX>
 inline __device__ void init_live_mlp(const RunDesc& R, float* xbuf, float* lbuf, char* msm, unsigned C, unsigned rank) {
   const int d = R.d, XS = mlp_xs(d);

@@ -913,10 +913,10 @@ inline __device__ void slice_walker_lanes(const LikParams& P, const SliceCfg& S,
   float* row = mem;
   float l = l0;
   int hlen = 0, flags = 0;
-  // evaluations, flushed to 64 bits once they pass 2^31 (a 64-bit count in the
-  // step's code: 16.6 against 16.0 ms for one walker's run at 2-D)
+  // (32 bits, as in slice_walker: 2^32 likelihoods of one walker take minutes
+  // even eight at a time; 64 bits in the step's code cost 4 % of one walker's
+  // run at 2-D, a flush once per step 2 %)
   unsigned evals = 0;
-  long long evals_far = 0;
   float r = 0.f, pre[kPreShrink] = {};
   auto fetch = [&](int s) {  // the row of step s, ahead of its use
     const float* src = dirs + (size_t)s * RW;
@@ -1106,17 +1106,12 @@ inline __device__ void slice_walker_lanes(const LikParams& P, const SliceCfg& S,
       }
       nsh += K;  // the same in every lane of the warp (K is)
     } while (__any_sync(kFull, open));
-    if (evals >> 31) {
-      evals_far += evals;
-      evals = 0;
-    }
   }
   if constexpr (!REG) __syncwarp();
   // the two sides' counts and flags
-  evals_far += evals;
-  const long long ev_r = __shfl_sync(kFull, evals_far, base + H);
+  const unsigned ev_r = __shfl_sync(kFull, evals, base + H);
   const int fl_r = __shfl_sync(kFull, flags, base + H);
-  evals_out = g == 0 ? evals_far + ev_r : 0;
+  evals_out = g == 0 ? (long long)evals + ev_r : 0;
   flags_out = g == 0 ? flags | fl_r : 0;
   if (active) {
     if constexpr (REG) {
